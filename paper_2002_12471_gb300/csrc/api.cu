@@ -89,6 +89,8 @@ void free_model(lmosem_ctx* c) {
     dev_free(c, &c->d_bpart_batch);
     dev_free(c, &c->d_weight);
     c->n_counts = 0.0;
+    if (c->terms_pending) c->terms_pending = c->terms_valid = false;  // their events are gone
+    c->use_grid = false;
     c->bpart_batch_floats = 0;
     c->batch_model = false;
     c->use_surrogate = false;
@@ -230,10 +232,16 @@ lmosem_status build_model_common(lmosem_ctx* c, const int32_t* d_angle, const fl
         free_model(c);
         return st;
     }
-    if ((st = sort_events(c, d_angle, d_u_mm, d_e_kev, n_events, n_subsets, h_offsets, n_real))) {
+    bool grid = false;
+    int64_t n_outside = 0;
+    if ((st = grid_plan(c, n_events, &grid)) ||
+        (st = sort_events(c, d_angle, d_u_mm, d_e_kev, n_events, n_subsets, h_offsets, n_real,
+                          grid ? &n_outside : nullptr))) {
         free_model(c);
         return st;
     }
+    // rows outside the grid's region cost about 30 times a path-sum row
+    c->use_grid = grid && n_outside <= n_events / 128;
     if ((st = sur ? build_checked_surrogate(c) : build_model_rows(c))) {
         free_model(c);
         return st;
@@ -278,7 +286,11 @@ lmosem_status lmosem_set_wait_budget(lmosem_ctx* c, int64_t cycles) {
 
 lmosem_status lmosem_model_terms(lmosem_ctx* c, int64_t* h_terms) {
     if (!c || !h_terms) return LMOSEM_EINVAL;
-    if (!c->terms_valid || !c->d_terms) return fail(c, LMOSEM_EINVAL, "no exact model build to count");
+    if (!c->terms_valid) return fail(c, LMOSEM_EINVAL, "no exact model build to count");
+    if (c->terms_pending) {
+        lmosem_status st = count_terms(c);
+        if (st) return st;
+    }
     unsigned long long v = 0;
     LMOSEM_CK(c, cudaMemcpyAsync(&v, c->d_terms, sizeof(v), cudaMemcpyDeviceToHost, c->stream));
     LMOSEM_CK(c, cudaStreamSynchronize(c->stream));
@@ -325,6 +337,7 @@ void lmosem_destroy(lmosem_ctx* c) {
     dev_free(c, &c->d_terms);
     dev_free(c, &c->d_status);
     dev_free(c, &c->d_surrogate);
+    grid_free(c);
     for (auto& r : c->prof) {
         cudaEventDestroy(r.a);
         cudaEventDestroy(r.b);
@@ -420,6 +433,7 @@ lmosem_status lmosem_create(const lmosem_object* obj, const lmosem_geometry* geo
             return LMOSEM_EINVAL;
         }
         mu[p] = (float)v;
+        c->mu_max = std::max(c->mu_max, v);
         bool sup = obj->h_support ? obj->h_support[p] != 0 : v > 0.0;
         if (sup) c->h_sup.push_back(p);
         if (v > 0.0) c->h_scat.push_back(p);
@@ -561,6 +575,10 @@ lmosem_status lmosem_build_model_binned(lmosem_ctx* c, const float* d_counts, in
         }
     }
     subset_row0[n_subsets] = r;
+    if (c->terms_pending) {  // the count of the last event list outlives it
+        lmosem_status st = count_terms(c);
+        if (st) return st;
+    }
     std::vector<int64_t> rank;  // ordinal of a positive bin in dense order -> row
     rank.reserve(n_rows);
     for (size_t q = 0; q < nbins; ++q)

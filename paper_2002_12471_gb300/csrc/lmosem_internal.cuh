@@ -27,6 +27,27 @@ constexpr int kTN = 128;
 constexpr int kMC = 32;
 constexpr int kBuildThreads = 256;
 
+// Grid of the scatter sum (grid.cu): its nodes, and per angle the scatter
+// pixels in subgroups of neighbouring positions.
+struct GridPlan {
+    int state = 0;               // 0: not made, 1: not usable for this problem, 2: ready
+    double hu = 0, rho_u = 0;    // step in u; in units of the interpolation kernel's width
+    double cut = 0;              // longest position cut (mm)
+    double u_lo = 0, x_lo = 0;   // first cell edge in u and in x = 2 sqrt(E / kappa)
+    int ncu = 0, nce = 0;        // cells
+    int nu = 0, ne = 0;          // nodes
+    double edge = 0, e_min = 0, e_max = 0;  // events beyond are summed directly
+    int max_sub = 0, n_sub = 0;  // subgroups per angle at most, and about
+    double strip = 0;            // share of the scatter pixels within an event's position cut
+    float log_g = 0, log_u = 0;  // log2 of the operands' scales
+    int32_t* d_slot_m = nullptr; // [a][subgroup][64]: scatter pixel or -1
+    int32_t* d_i0 = nullptr;     // [a][subgroup]: first node
+    int32_t* d_n_sub = nullptr;  // [a]
+    float2* d_urange = nullptr;  // [a]: positions of the outermost scatter pixels
+    float4* d_enode = nullptr;   // energies of the node pairs
+    int32_t* d_angle_slot = nullptr;  // [a]: place of the angle in the sorted order
+};
+
 }  // namespace lmosem
 
 struct lmosem_ctx {
@@ -46,6 +67,7 @@ struct lmosem_ctx {
 
     int n_sup = 0, n_scat = 0, ld_w = 0;  // ld_w: support padded to kTN
     std::vector<int32_t> h_sup, h_scat;
+    double mu_max = 0;    // largest entry of the mu-map
     double kbar = 0;      // circle mean of the Klein-Nishina shape at E0
     double de0 = 0;       // energy-window mass of the photopeak
 
@@ -106,6 +128,9 @@ struct lmosem_ctx {
     double* d_scalar = nullptr;   // small FP64 scratch
     unsigned long long* d_terms = nullptr;  // path terms of the last model build (path-sum kernels)
     bool terms_valid = false;
+    bool terms_pending = false;   // the last build used the grid: the terms are counted when asked for
+    lmosem::GridPlan grid;
+    bool use_grid = false;        // the model's exact rows come from the grid
     int* d_status = nullptr;      // [0] = 1 after a bounded device wait ran out
     long long wait_budget = 2000000000LL;  // clock cycles per bounded wait
     int pass_variant = 0;         // 0 auto, 1 register pipeline, 2 bulk-copy ring, 3 cp.async ring,
@@ -282,15 +307,28 @@ __device__ __forceinline__ float sum8_in_order(const float* v) {
 lmosem_status build_tables(lmosem_ctx* c);                      // siddon.cu
 // h_offsets: n_real + 1 event offsets of the realisations (nullptr: one)
 // EINVAL unless every event's angle, position and energy are in range (synchronises)
+// (n_outside != nullptr: also the events outside the grid's region)
 lmosem_status validate_events(lmosem_ctx* c, const int32_t* d_angle, const float* d_u, const float* d_e,
-                              int64_t n);
+                              int64_t n, int64_t* n_outside = nullptr);
 // support.cu: the binned-OSEM support initialiser
 lmosem_status run_binned_support(lmosem_ctx* c, const int32_t* d_angle, const float* d_u, int64_t n,
                                  int n_subsets, int n_iters, double threshold, int dilate,
                                  uint8_t* h_support, float* d_image);
 lmosem_status sort_events(lmosem_ctx* c, const int32_t* d_angle, const float* d_u,
                           const float* d_e, int64_t n, int n_subsets,
-                          const int64_t* h_offsets, int n_real);  // sort.cu
+                          const int64_t* h_offsets, int n_real, int64_t* n_outside = nullptr);  // sort.cu
+// exclusive prefix sum in place; tot: scan_blocks(n) words of scratch
+int64_t scan_blocks(int64_t n);
+lmosem_status exclusive_scan(lmosem_ctx* c, int32_t* x, int64_t n, int32_t* tot);
+// grid.cu
+lmosem_status grid_plan(lmosem_ctx* c, int64_t n_events, bool* use);
+void grid_free(lmosem_ctx* c);
+lmosem_status grid_count_outside(lmosem_ctx* c, const int32_t* a, const float* u, const float* e, int64_t n,
+                                 int32_t* d_n);
+lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& slot_angle);
+// model.cu: staged FP32 rows (d_stage) to the scaled rows row0 ..; path terms of the current events
+lmosem_status quantize_rows(lmosem_ctx* c, int64_t rows, int64_t row0);
+lmosem_status count_terms(lmosem_ctx* c);
 lmosem_status build_model_rows(lmosem_ctx* c);
 // binned rows: model of every (angle, position bin, energy bin) row of the
 // row map ([a][b][k] -> sorted row or -1) with energy bin edges e_edges

@@ -1148,6 +1148,22 @@ lmosem_status wtab_all_with_sens(lmosem_ctx* c, double* sens_angle, float w_cons
     return LMOSEM_OK;
 }
 
+lmosem_status quantize_rows(lmosem_ctx* c, int64_t rows, int64_t row0) {
+    const int qthreads = 256;
+    const unsigned qblocks = (unsigned)((rows + qthreads / 32 - 1) / (qthreads / 32));
+    LMOSEM_PROF_BEGIN(c);
+    if (c->fmt == LMOSEM_MODEL_FP16_SCALED)
+        k_quantize<__half><<<qblocks, qthreads, 0, c->stream>>>(c->d_stage, c->ld_model, rows, c->n_sup, c->ld_model,
+                                                                reinterpret_cast<__half*>(c->d_model), row0,
+                                                                c->d_scale, 32768.0f);
+    else
+        k_quantize<__nv_bfloat16><<<qblocks, qthreads, 0, c->stream>>>(
+            c->d_stage, c->ld_model, rows, c->n_sup, c->ld_model, reinterpret_cast<__nv_bfloat16*>(c->d_model), row0,
+            c->d_scale, 1.0f);
+    LMOSEM_LAUNCHED(c, LMOSEM_K_QUANTIZE);
+    return LMOSEM_OK;
+}
+
 lmosem_status build_model_rows(lmosem_ctx* c) {
     if (c->use_surrogate) {
         dev_free(c, &c->d_wtab_all);  // the surrogate form has no use for the tables
@@ -1165,6 +1181,12 @@ lmosem_status build_model_rows(lmosem_ctx* c) {
         if (a < c->n_angles) slot_angle.push_back(a);
     }
     const int ns = (int)slot_angle.size();
+    if (c->use_grid && !c->scatter_only) {
+        dev_free(c, &c->d_wtab_all);  // the grid has tables of its own
+        c->terms_valid = c->terms_pending = true;
+        return build_model_rows_grid(c, slot_angle);
+    }
+    c->terms_pending = false;
 
     // angle groups bounded by the scatter-table budget (three FP32 planes);
     // one group indexed by angle when the sensitivity pass left every
@@ -1325,20 +1347,7 @@ lmosem_status build_model_rows(lmosem_ctx* c) {
                 k_pathsum_narrow<<<(unsigned)tiles, kBuildThreads, smem_n, c->stream>>>(P);
             LMOSEM_LAUNCHED(c, LMOSEM_K_PATHSUM);
         }
-        if (scaled) {
-            const int qthreads = 256;
-            unsigned qblocks = (unsigned)((grows + qthreads / 32 - 1) / (qthreads / 32));
-            LMOSEM_PROF_BEGIN(c);
-            if (c->fmt == LMOSEM_MODEL_FP16_SCALED)
-                k_quantize<__half><<<qblocks, qthreads, 0, c->stream>>>(
-                    c->d_stage, c->ld_model, grows, c->n_sup, c->ld_model,
-                    reinterpret_cast<__half*>(c->d_model), grow0, c->d_scale, 32768.0f);
-            else
-                k_quantize<__nv_bfloat16><<<qblocks, qthreads, 0, c->stream>>>(
-                    c->d_stage, c->ld_model, grows, c->n_sup, c->ld_model,
-                    reinterpret_cast<__nv_bfloat16*>(c->d_model), grow0, c->d_scale, 1.0f);
-            LMOSEM_LAUNCHED(c, LMOSEM_K_QUANTIZE);
-        }
+        if (scaled && (st = quantize_rows(c, grows, grow0))) return st;
     }
     // stream-ordered frees: no host wait (the caller's events were consumed
     // before the sort's last synchronisation)
@@ -1398,7 +1407,96 @@ __global__ void __launch_bounds__(256) k_judge_rows(const float* __restrict__ mo
     }
 }
 
+
+// Path terms of sorted rows [row0, row0 + cnt) of one angle: one per (event,
+// column) and one per (event, column, scatter pixel) inside both cuts
+struct TermArgs {
+    const float* u_s;
+    const float* e_s;
+    const int64_t* ent;          // (angle, plane slot, first row, rows) per entry
+    const float4* mpar;
+    const uint2* hull;
+    int n_scat, n_ptiles, n_sup, e_cut;
+    unsigned long long* n_terms;
+};
+__global__ void __launch_bounds__(256) k_count_terms(TermArgs A) {
+    __shared__ float su[kTJ], se[kTJ];
+    const int64_t* en = A.ent + 4 * blockIdx.x;
+    const float4* mp = A.mpar + (size_t)en[0] * A.n_scat;
+    const uint2* hull = A.hull + (size_t)en[1] * A.n_ptiles * A.n_scat;
+    unsigned long long n = 0;
+    for (int64_t r0 = (int64_t)blockIdx.y * kTJ; r0 < en[3]; r0 += (int64_t)gridDim.y * kTJ) {
+        const int nr = (int)min((int64_t)kTJ, en[3] - r0);
+        __syncthreads();
+        if (threadIdx.x < nr) {
+            su[threadIdx.x] = A.u_s[en[2] + r0 + threadIdx.x];
+            se[threadIdx.x] = A.e_s[en[2] + r0 + threadIdx.x];
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) n += (unsigned long long)nr * A.n_sup;
+        for (int m = threadIdx.x; m < A.n_scat; m += blockDim.x) {
+            const float4 q = mp[m];
+            for (int j = 0; j < nr; ++j) {
+                if (!(fabsf(su[j] - q.x) <= q.w)) continue;
+                for (int pt = 0; pt < A.n_ptiles; ++pt)
+                    if (!(A.e_cut && energy_cut(se[j], hull[(size_t)pt * A.n_scat + m])))
+                        n += (unsigned)min(kTN, A.n_sup - pt * kTN);
+            }
+        }
+    }
+    for (int o = 16; o; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(A.n_terms, n);
+}
+
 }  // namespace
+
+// Path terms of the current events (rows built on the grid are no sums of
+// terms; the count stays that of the sum they evaluate)
+lmosem_status count_terms(lmosem_ctx* c) {
+    lmosem_status st;
+    if (!c->d_terms && (st = dev_alloc(c, &c->d_terms, 1))) return st;
+    LMOSEM_CK(c, cudaMemsetAsync(c->d_terms, 0, sizeof(unsigned long long), c->stream));
+    const int na = c->n_angles;
+    const int gsz = (int)std::max<int64_t>(
+        1, std::min<int64_t>(na, c->table_budget / (wtab_angle_floats(c) * (int64_t)sizeof(float))));
+    std::vector<int32_t> ident(na);
+    std::vector<int64_t> ent, first(1, 0);
+    for (int a = 0; a < na; ++a) ident[a] = a;
+    for (int a0 = 0; a0 < na; a0 += gsz) {
+        for (int a = a0; a < std::min(na, a0 + gsz); ++a)
+            for (int r = 0; r < c->n_real; ++r) {
+                const size_t k = (size_t)r * na + a;
+                if (c->h_angle_cnt[k] > 0) ent.insert(ent.end(), {a, a - a0, c->h_angle_row0[k], c->h_angle_cnt[k]});
+            }
+        first.push_back((int64_t)ent.size() / 4);
+    }
+    int32_t* d_ang = nullptr;
+    int64_t* d_ent = nullptr;
+    float* wtab = nullptr;
+    Scratch tmp(c);
+    if ((st = tmp.alloc(&d_ang, na)) || (st = tmp.alloc(&d_ent, ent.size())) ||
+        (st = tmp.alloc(&wtab, (size_t)gsz * wtab_angle_floats(c))))
+        return st;
+    LMOSEM_CK(c, cudaMemcpyAsync(d_ang, ident.data(), na * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
+    LMOSEM_CK(c, cudaMemcpyAsync(d_ent, ent.data(), ent.size() * sizeof(int64_t), cudaMemcpyHostToDevice, c->stream));
+    for (int gi = 0; gi * gsz < na; ++gi) {
+        const int64_t n_ent = first[gi + 1] - first[gi];
+        if (n_ent == 0) continue;
+        const int n = std::min(gsz, na - gi * gsz);
+        WTabArgs W = wtab_args(c, wtab, gsz, d_ang, gi * gsz);
+        if ((st = hull_reset(c, W, n))) return st;
+        LMOSEM_PROF_BEGIN(c);
+        k_wtable<<<dim3((c->ld_w + 255) / 256, c->n_scat), 256, 0, c->stream>>>(W, n);
+        LMOSEM_LAUNCHED(c, LMOSEM_K_WTABLE);
+        TermArgs T{c->d_u_s, c->d_e_s, d_ent + 4 * first[gi], c->d_mpar, W.hull, c->n_scat, W.n_ptiles, c->n_sup,
+                   c->e_sigma > 0.0f ? 1 : 0, c->d_terms};
+        LMOSEM_PROF_BEGIN(c);
+        k_count_terms<<<dim3((unsigned)n_ent, 32), 256, 0, c->stream>>>(T);
+        LMOSEM_LAUNCHED(c, LMOSEM_K_OTHER);
+    }
+    c->terms_pending = false;
+    return LMOSEM_OK;
+}
 
 // Exact FP32 rows (primary and every first-order scatter path) of K sorted
 // model rows h_rows (increasing; d_rows their device copy) into d_out
@@ -1406,10 +1504,11 @@ __global__ void __launch_bounds__(256) k_judge_rows(const float* __restrict__ mo
 // sum in place of the model's events, and the model's event state is put back
 // after.  The rows of a (realisation, angle) stay contiguous in the sample,
 // and a row's bits do not depend on the other events of its tiles, so every
-// row equals the one the exact build of all events gives.  h_e (K floats, may
-// be NULL) receives the rows' event energies.
+// row equals the one the exact build of all events gives (as_model: formed
+// as that build forms them, on the grid or path by path; else path by path).
+// h_e (K floats, may be NULL) receives the rows' event energies.
 lmosem_status exact_rows(lmosem_ctx* c, const std::vector<int64_t>& h_rows, const int64_t* d_rows, float* d_out,
-                         float* h_e) {
+                         float* h_e, bool as_model) {
     const int64_t K = (int64_t)h_rows.size();
     if (K == 0) return LMOSEM_OK;
     lmosem_status st;
@@ -1450,7 +1549,11 @@ lmosem_status exact_rows(lmosem_ctx* c, const std::vector<int64_t>& h_rows, cons
     c->d_model = d_out;
     c->fmt = LMOSEM_MODEL_FP32;
     c->use_surrogate = false;
+    const bool grid0 = c->use_grid;
+    c->use_grid = c->use_grid && as_model;
     st = build_model_rows(c);
+    if (!st && c->terms_pending) st = count_terms(c);  // while these events are in place
+    c->use_grid = grid0;
     c->use_surrogate = sur0;
     c->fmt = fmt0;
     c->d_model = m0;
@@ -1503,7 +1606,7 @@ lmosem_status judge_surrogate(lmosem_ctx* c, double* rel_err, double* row_max, s
         return st;
     LMOSEM_CK(c, cudaMemcpyAsync(d_rows, rows.data(), K * sizeof(int64_t), cudaMemcpyHostToDevice, c->stream));
     std::vector<float> energies(K);
-    if ((st = exact_rows(c, rows, d_rows, d_ex, energies.data()))) return st;
+    if ((st = exact_rows(c, rows, d_rows, d_ex, energies.data(), false))) return st;
     LMOSEM_PROF_BEGIN(c);
     k_judge_rows<<<(unsigned)K, 256, 0, c->stream>>>(reinterpret_cast<const float*>(c->d_model), c->ld_model,
                                                       d_rows, d_ex, c->n_sup, d_sums);
@@ -1576,7 +1679,7 @@ lmosem_status rebuild_rows_below(lmosem_ctx* c, double e_cut, int64_t* n_rebuilt
         const int64_t K = std::min<int64_t>(per, (int64_t)rows.size() - k0);
         std::vector<int64_t> part(rows.begin() + k0, rows.begin() + k0 + K);
         LMOSEM_CK(c, cudaMemcpyAsync(d_rows, part.data(), K * sizeof(int64_t), cudaMemcpyHostToDevice, c->stream));
-        if ((st = exact_rows(c, part, d_rows, d_ex, nullptr))) return st;
+        if ((st = exact_rows(c, part, d_rows, d_ex, nullptr, true))) return st;
         LMOSEM_PROF_BEGIN(c);
         k_scatter_rows<<<(unsigned)K, 256, 0, c->stream>>>(reinterpret_cast<const float4*>(d_ex), d_rows,
                                                            c->ld_model / 4, reinterpret_cast<float4*>(c->d_model));

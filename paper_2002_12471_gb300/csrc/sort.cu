@@ -179,23 +179,34 @@ __global__ void k_gather_events(const int32_t* __restrict__ perm, int64_t n,
     rank[j] = r;
 }
 
+}  // namespace
+
+int64_t scan_blocks(int64_t n) { return (n + kScanBlock * 4 - 1) / (kScanBlock * 4); }
+
+lmosem_status exclusive_scan(lmosem_ctx* c, int32_t* x, int64_t n, int32_t* tot) {
+    const int sblk = (int)scan_blocks(n);
+    LMOSEM_PROF_BEGIN(c);
+    k_scan_local<<<sblk, kScanBlock, 0, c->stream>>>(x, n, tot);
+    LMOSEM_LAUNCHED(c, LMOSEM_K_SORT);
+    LMOSEM_PROF_BEGIN(c);
+    k_scan_totals<<<1, kScanBlock, 0, c->stream>>>(tot, sblk);
+    LMOSEM_LAUNCHED(c, LMOSEM_K_SORT);
+    LMOSEM_PROF_BEGIN(c);
+    k_scan_add<<<(int)((n + 255) / 256), 256, 0, c->stream>>>(x, n, tot);
+    LMOSEM_LAUNCHED(c, LMOSEM_K_SORT);
+    return LMOSEM_OK;
+}
+
+namespace {
+
 lmosem_status counting_pass(lmosem_ctx* c, const Digit& dg, int ndig, const int32_t* perm_in,
                             int32_t* perm_out, int64_t n, int32_t* H, int32_t* tot) {
     int nblk = (int)((n + kSortThreads - 1) / kSortThreads);
     LMOSEM_PROF_BEGIN(c);
     k_hist<<<nblk, kSortThreads, ndig * sizeof(int32_t), c->stream>>>(dg, perm_in, n, ndig, H);
     LMOSEM_LAUNCHED(c, LMOSEM_K_SORT);
-    int64_t hn = (int64_t)ndig * nblk;
-    int sblk = (int)((hn + kScanBlock * 4 - 1) / (kScanBlock * 4));
-    LMOSEM_PROF_BEGIN(c);
-    k_scan_local<<<sblk, kScanBlock, 0, c->stream>>>(H, hn, tot);
-    LMOSEM_LAUNCHED(c, LMOSEM_K_SORT);
-    LMOSEM_PROF_BEGIN(c);
-    k_scan_totals<<<1, kScanBlock, 0, c->stream>>>(tot, sblk);
-    LMOSEM_LAUNCHED(c, LMOSEM_K_SORT);
-    LMOSEM_PROF_BEGIN(c);
-    k_scan_add<<<(int)((hn + 255) / 256), 256, 0, c->stream>>>(H, hn, tot);
-    LMOSEM_LAUNCHED(c, LMOSEM_K_SORT);
+    lmosem_status st;
+    if ((st = exclusive_scan(c, H, (int64_t)ndig * nblk, tot))) return st;
     size_t smem = (size_t)(kSortThreads / 32) * ndig * sizeof(int32_t);
     LMOSEM_PROF_BEGIN(c);
     k_scatter<<<nblk, kSortThreads, smem, c->stream>>>(dg, perm_in, n, ndig, H, perm_out);
@@ -206,20 +217,23 @@ lmosem_status counting_pass(lmosem_ctx* c, const Digit& dg, int ndig, const int3
 }  // namespace
 
 lmosem_status validate_events(lmosem_ctx* c, const int32_t* d_angle, const float* d_u, const float* d_e,
-                              int64_t n) {
+                              int64_t n, int64_t* n_outside) {
     lmosem_status st;
     const float half = (float)(0.5 * c->n_bins * c->bin_mm);
     int32_t* d_bad = nullptr;
     Scratch tmp(c);
-    if ((st = tmp.alloc(&d_bad, 1))) return st;
-    LMOSEM_CK(c, cudaMemsetAsync(d_bad, 0, sizeof(int32_t), c->stream));
+    if ((st = tmp.alloc(&d_bad, 2))) return st;
+    LMOSEM_CK(c, cudaMemsetAsync(d_bad, 0, 2 * sizeof(int32_t), c->stream));
     LMOSEM_PROF_BEGIN(c);
     k_check_events<<<(int)((n + 255) / 256), 256, 0, c->stream>>>(
         d_angle, d_u, d_e, n, c->n_angles, half, (float)c->e_lo, (float)c->e_hi, d_bad);
     LMOSEM_LAUNCHED(c, LMOSEM_K_SORT);
-    int32_t bad = 0;
-    LMOSEM_CK(c, cudaMemcpyAsync(&bad, d_bad, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
+    if (n_outside && (st = grid_count_outside(c, d_angle, d_u, d_e, n, d_bad + 1))) return st;
+    int32_t h[2] = {0, 0};
+    LMOSEM_CK(c, cudaMemcpyAsync(h, d_bad, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
     LMOSEM_CK(c, cudaStreamSynchronize(c->stream));
+    const int32_t bad = h[0];
+    if (n_outside) *n_outside = h[1];
     if (bad) return fail(c, LMOSEM_EINVAL, std::to_string(bad) +
                                                " events have an angle, position or energy out of range");
     return LMOSEM_OK;
@@ -227,9 +241,9 @@ lmosem_status validate_events(lmosem_ctx* c, const int32_t* d_angle, const float
 
 lmosem_status sort_events(lmosem_ctx* c, const int32_t* d_angle, const float* d_u,
                           const float* d_e, int64_t n, int n_subsets, const int64_t* h_offsets,
-                          int n_real) {
+                          int n_real, int64_t* n_outside) {
     lmosem_status st;
-    if ((st = validate_events(c, d_angle, d_u, d_e, n))) return st;
+    if ((st = validate_events(c, d_angle, d_u, d_e, n, n_outside))) return st;
     const float half = (float)(0.5 * c->n_bins * c->bin_mm);
 
     const int group = (c->n_angles + n_subsets - 1) / n_subsets;
