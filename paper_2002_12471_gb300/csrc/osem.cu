@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kMaxPassThreads, pass_min_ctas<H, VPT>()) k_pa
             const bool ok = r + i < re && y > 0.0f;
             if constexpr (BACK) {
                 float inv = ok ? 1.0f / y : 0.0f;
-                if constexpr (W) inv *= A.weight[r + i];  // a binned row counts its photons
+                if constexpr (W) inv *= ok ? A.weight[r + i] : 0.0f;  // a binned row counts its photons
                 const float2 inv2 = make_float2(inv, inv);
 #pragma unroll
                 for (int v = 0; v < VPT; ++v) {
@@ -442,7 +442,7 @@ __global__ void __launch_bounds__(kMaxPassThreads, pass_min_ctas<H, VPT>()) k_pa
             const bool ok = r + i < re && y > 0.0f;
             if constexpr (BACK) {
                 float inv = ok ? 1.0f / y : 0.0f;
-                if constexpr (W) inv *= A.weight[r + i];
+                if constexpr (W) inv *= ok ? A.weight[r + i] : 0.0f;
                 const float2 inv2 = make_float2(inv, inv);
 #pragma unroll
                 for (int v = 0; v < VPT; ++v) {
