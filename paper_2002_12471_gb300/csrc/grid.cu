@@ -299,17 +299,6 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
 
-// one lane of a converged warp.  The products are issued under this predicate
-// and not under lane == 0: the compiler then knows that a single thread is
-// active and keeps the operands in uniform registers.  Measured for a unit of
-// three M = 128, N = 112 products: 213 cycles under lane == 0, 168 (the tensor
-// core's rate) under elect.sync, and 430 against 180 beside busy warps.
-__device__ __forceinline__ bool elect_one() {
-    uint32_t p;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-    return p != 0;
-}
-
 __device__ __forceinline__ void tmem_st16(uint32_t a, const uint32_t (&r)[16]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n" ::"r"(a),

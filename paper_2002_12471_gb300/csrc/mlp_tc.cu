@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_tc(TcArgs A) {
 
     if (warp == kProdWarp) {
         // ---------------- producer: inputs of a pair, then its weight chunks in product order
-        if (lane == 0) {
+        if (elect_one()) {
             bool ok = true;
             auto load_x = [&](int g, int64_t p) -> bool {
                 if (2 * p + g >= nj) return true;
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_tc(TcArgs A) {
         __syncwarp();
     } else if (warp == kMmaWarp) {
         // ---------------- MMA issuer: layer by layer, alternating between the pair's tiles
-        if (lane == 0) {
+        if (elect_one()) {
             bool ok = true;
             uint32_t n = 0;  // weight chunks consumed
             for (int64_t p = 0; p < npairs && ok; ++p) {
@@ -421,11 +421,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_tc(TcArgs A) {
     }
     __syncthreads();
     if (*abort_flag) {
-        if (warp == kMmaWarp && lane == 0) {  // products in flight finish before TMEM is freed
+        if (warp == kMmaWarp && elect_one()) {  // products in flight finish before TMEM is freed
             mma_commit(drain);
             bar_wait(drain, 0u, kDrainCycles, nullptr);
         }
-        if (warp == kProdWarp && lane == 0) {  // and the last copy of every slot lands
+        if (warp == kProdWarp && nw + nx0 + nx1 > 0) {  // (the lane that issued them) and the last copy of every slot lands
             for (uint32_t sl = 0; sl < (uint32_t)kSlots; ++sl) {
                 const uint32_t u = nw / kSlots + (sl < nw % kSlots ? 1u : 0u);
                 if (u > 0) bar_wait(&wfull[sl], (u - 1) & 1u, kDrainCycles, nullptr);
@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(128) k_gemm_tc(GemmTcArgs G) {
         cp_wait_upto(issued - c - 1);  // chunk c's copies (this thread's) have landed
         fence_async_smem();            // and are visible to the tensor core
         __syncthreads();
-        if (tid == 0) {
+        if (warp == 0 && elect_one()) {
             fence_after();
             const uint32_t a_s = base + (uint32_t)buf * kStage, b_s = a_s + kAStage;
             const int nmma = min(2, (ke - (kb + c * kGemmChunk) + 15) / 16);
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(128) k_gemm_tc(GemmTcArgs G) {
         }
     }
     if (!ok) asm volatile("cp.async.wait_group 0;\n" ::: "memory");  // no copy outlives the CTA
-    if (tid == 0) {
+    if (warp == 0 && elect_one()) {  // (the lane that issued the products)
         mma_commit(&bars[S]);  // every product issued so far
         s_ok = bar_wait(&bars[S], 0u, ok ? G.budget : kDrainCycles, nullptr) && ok;
         if (!s_ok) atomicExch(G.status, 1);
