@@ -297,58 +297,131 @@ __global__ void k_target_floor(const float* __restrict__ t, int64_t n, float flo
     if (threadIdx.x == 0) *floor = fl;
 }
 
-// mean and standard deviation of the (floored) targets minus the baseline
-// (FP64, one block, fixed order) into the blob's mu and sigma
-__global__ void k_target_stats(const float* __restrict__ t, const float* __restrict__ feat, int64_t n,
-                               const float* __restrict__ floor, float* __restrict__ blob) {
-    __shared__ double s1[256], s2[256];
+// The one-off sums of a training run (2M samples: 25 ms in single blocks and
+// in one block per entry of the normal matrix, 0.9 ms as below).  Each block
+// sums its share of the rows in FP64 and leaves a partial sum; the partial
+// sums are added in block order, so the result is a function of the input.
+constexpr int kSetupBlocks = 304, kSetupThreads = 256;
+
+__device__ __forceinline__ void setup_rows(int64_t n, int64_t* r0, int64_t* r1) {
+    const int64_t per = (n + gridDim.x - 1) / gridDim.x;
+    *r0 = min(n, per * blockIdx.x);
+    *r1 = min(n, *r0 + per);
+}
+
+// sums of the (floored) targets minus the baseline and of their squares
+__global__ void __launch_bounds__(kSetupThreads) k_target_sums(const float* __restrict__ t,
+                                                               const float* __restrict__ feat, int64_t n,
+                                                               const float* __restrict__ floor,
+                                                               const float* __restrict__ blob,
+                                                               double* __restrict__ part) {
+    __shared__ double s1[kSetupThreads], s2[kSetupThreads];
     const float fl = *floor;
+    int64_t r0, r1;
+    setup_rows(n, &r0, &r1);
     double a = 0.0, b = 0.0;
-    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int64_t i = r0 + threadIdx.x; i < r1; i += kSetupThreads) {
         const double ti = fmaxf(t[i], fl) - baseline(blob, feat + i * kIn);
         a += ti;
         b += ti * ti;
     }
     s1[threadIdx.x] = a;
     s2[threadIdx.x] = b;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double A = 0.0, Bq = 0.0;
-        for (int k = 0; k < (int)blockDim.x; ++k) {
-            A += s1[k];
-            Bq += s2[k];
+    for (int o = kSetupThreads / 2; o; o >>= 1) {
+        __syncthreads();
+        if (threadIdx.x < o) {
+            s1[threadIdx.x] += s1[threadIdx.x + o];
+            s2[threadIdx.x] += s2[threadIdx.x + o];
         }
-        const double mu = A / n;
-        const double var = fmax(Bq / n - mu * mu, 1e-12);
-        blob[kOffMu] = (float)mu;
-        blob[kOffSigma] = (float)sqrt(var);
     }
+    if (threadIdx.x == 0) {
+        part[2 * blockIdx.x] = s1[0];
+        part[2 * blockIdx.x + 1] = s2[0];
+    }
+}
+// their mean and standard deviation into the blob's mu and sigma
+__global__ void k_target_stats(const double* __restrict__ part, int nparts, int64_t n, float* __restrict__ blob) {
+    if (threadIdx.x != 0) return;
+    double a = 0.0, b = 0.0;
+    for (int k = 0; k < nparts; ++k) {
+        a += part[2 * k];
+        b += part[2 * k + 1];
+    }
+    const double mu = a / n;
+    blob[kOffMu] = (float)mu;
+    blob[kOffSigma] = (float)sqrt(fmax(b / n - mu * mu, 1e-12));
 }
 
 // least squares of the baseline: for m rows evenly spaced over the samples,
-// block (i, j) (j <= i) sums phi_i phi_j and block (i, kBasis) sums phi_i t
-// (floored), FP64 in a fixed order
-__global__ void k_basis_normal(const float* __restrict__ feat, const float* __restrict__ t, int64_t n, int64_t m,
-                               const float* __restrict__ floor, double* __restrict__ out /* kBasis x (kBasis+1) */) {
-    const int bi = blockIdx.x, bj = blockIdx.y;
-    if (bj < kBasis && bj > bi) return;
-    __shared__ double sh[256];
+// the sums phi_i phi_j (j <= i) and phi_i t (floored; j = kBasis).  A block
+// stages the basis of kNormalRows rows in shared memory (every entry of a row
+// is then formed once); thread k sums the entries k, k + blockDim.x of the
+// lower triangle.
+constexpr int kNormalRows = 64, kNormalEntries = kBasis * (kBasis + 1) / 2 + kBasis;
+__global__ void __launch_bounds__(kSetupThreads) k_basis_normal(const float* __restrict__ feat,
+                                                                const float* __restrict__ t, int64_t n, int64_t m,
+                                                                const float* __restrict__ floor,
+                                                                double* __restrict__ part /* [block][entry] */) {
+    static_assert(kNormalEntries <= 2 * kSetupThreads, "two entries per thread");
+    __shared__ float sphi[kNormalRows][kBasis + 1];
     const float fl = *floor;
-    double acc = 0.0;
-    for (int64_t r = threadIdx.x; r < m; r += blockDim.x) {
-        const int64_t i = (int64_t)((double)r * (double)n / (double)m);
-        float phi[kBasis];
-        basis(feat + i * kIn, phi);
-        const double pj = bj < kBasis ? (double)phi[bj] : (double)fmaxf(t[i], fl);
-        acc += (double)phi[bi] * pj;
+    int ei[2], ej[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int k = threadIdx.x + e * kSetupThreads;
+        int i = 0, j = 0;
+        if (k < kNormalEntries - kBasis) {
+            while ((i + 1) * (i + 2) / 2 <= k) ++i;
+            j = k - i * (i + 1) / 2;
+        } else if (k < kNormalEntries) {
+            i = k - (kNormalEntries - kBasis);
+            j = kBasis;
+        }
+        ei[e] = i;
+        ej[e] = j;
     }
-    sh[threadIdx.x] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int k = 0; k < (int)blockDim.x; ++k) s += sh[k];
-        out[bi * (kBasis + 1) + bj] = s;
+    int64_t r0, r1;
+    setup_rows(m, &r0, &r1);
+    double acc[2] = {0.0, 0.0};
+    for (int64_t b = r0; b < r1; b += kNormalRows) {
+        const int nr = (int)min((int64_t)kNormalRows, r1 - b);
+        __syncthreads();
+        if ((int)threadIdx.x < nr) {
+            const int64_t i = (int64_t)((double)(b + threadIdx.x) * (double)n / (double)m);
+            float phi[kBasis];
+            basis(feat + i * kIn, phi);
+#pragma unroll
+            for (int k = 0; k < kBasis; ++k) sphi[threadIdx.x][k] = phi[k];
+            sphi[threadIdx.x][kBasis] = fmaxf(t[i], fl);
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int r = 0; r < nr; ++r) {
+            acc[0] += (double)sphi[r][ei[0]] * (double)sphi[r][ej[0]];
+            acc[1] += (double)sphi[r][ei[1]] * (double)sphi[r][ej[1]];
+        }
     }
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int k = threadIdx.x + e * kSetupThreads;
+        if (k < kNormalEntries) part[(size_t)blockIdx.x * kNormalEntries + k] = acc[e];
+    }
+}
+__global__ void k_basis_normal_sum(const double* __restrict__ part, int nparts,
+                                   double* __restrict__ out /* kBasis x (kBasis+1) */) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= kNormalEntries) return;
+    double s = 0.0;
+#pragma unroll 8
+    for (int b = 0; b < nparts; ++b) s += part[(size_t)b * kNormalEntries + k];
+    int i = 0, j = kBasis;
+    if (k < kNormalEntries - kBasis) {
+        while ((i + 1) * (i + 2) / 2 <= k) ++i;
+        j = k - i * (i + 1) / 2;
+    } else {
+        i = k - (kNormalEntries - kBasis);
+    }
+    out[i * (kBasis + 1) + j] = s;
 }
 
 // ---------------------------------------------------------------- features
@@ -520,24 +593,60 @@ __global__ void k_cdf_chunks(const float* __restrict__ rel, int64_t n, float alp
         csum[blockIdx.x] = s;
     }
 }
-__global__ void k_cdf_offsets(double* __restrict__ csum, int64_t nchunks) {
-    if (threadIdx.x != 0) return;
-    double acc = 0.0;  // exclusive scan in place
-    for (int64_t k = 0; k < nchunks; ++k) {
-        const double v = csum[k];
-        csum[k] = acc;
-        acc += v;
+// exclusive scan of the chunk sums in place, in order (one block: a tile of
+// chunks at a time through shared memory)
+__global__ void __launch_bounds__(1024) k_cdf_offsets(double* __restrict__ csum, int64_t nchunks) {
+    __shared__ double sh[1024];
+    __shared__ double carry;
+    if (threadIdx.x == 0) carry = 0.0;
+    for (int64_t b = 0; b < nchunks; b += 1024) {
+        __syncthreads();
+        if (b + threadIdx.x < nchunks) sh[threadIdx.x] = csum[b + threadIdx.x];
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double acc = carry;
+            const int m = (int)min((int64_t)1024, nchunks - b);
+            for (int k = 0; k < m; ++k) {
+                const double v = sh[k];
+                sh[k] = acc;
+                acc += v;
+            }
+            carry = acc;
+        }
+        __syncthreads();
+        if (b + threadIdx.x < nchunks) csum[b + threadIdx.x] = sh[threadIdx.x];
     }
 }
-__global__ void k_cdf_fill(const float* __restrict__ rel, int64_t n, float alpha, const double* __restrict__ off,
-                           double* __restrict__ cdf) {
-    if (threadIdx.x != 0) return;  // one thread per chunk, in order
-    const int64_t c0 = (int64_t)blockIdx.x * kCdfChunk;
-    double acc = off[blockIdx.x];
-    for (int64_t i = c0; i < min(n, c0 + kCdfChunk); ++i) {
-        acc += exp((double)alpha * rel[i]);
-        cdf[i] = acc;
+// a block per chunk: each thread sums kCdfChunk / 256 consecutive weights, one
+// thread scans the 256 sums in order, and each writes its prefix sums from its
+// offset (its last value is the next thread's offset: they never decrease)
+__global__ void __launch_bounds__(256) k_cdf_fill(const float* __restrict__ rel, int64_t n, float alpha,
+                                                  const double* __restrict__ off, double* __restrict__ cdf) {
+    constexpr int kPer = kCdfChunk / 256;
+    __shared__ double sh[256];
+    const int64_t i0 = (int64_t)blockIdx.x * kCdfChunk + threadIdx.x * kPer;
+    double w[kPer];
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        if (i0 + k < n) s += exp((double)alpha * rel[i0 + k]);
+        w[k] = s;
     }
+    sh[threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double acc = off[blockIdx.x];
+        for (int k = 0; k < 256; ++k) {
+            const double v = sh[k];
+            sh[k] = acc;
+            acc += v;
+        }
+    }
+    __syncthreads();
+    const double o = sh[threadIdx.x];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k)
+        if (i0 + k < n) cdf[i0 + k] = o + w[k];
 }
 
 // surrogate inputs of rows [r0, r0 + nrows) x all support pixels, BF16; with
@@ -773,10 +882,16 @@ lmosem_status fit_baseline(lmosem_ctx* c, const float* feat, const float* targ, 
         double* d_ne = nullptr;
         Scratch tmp(c);
         lmosem_status st;
-        if ((st = tmp.alloc(&d_ne, (size_t)kBasis * (kBasis + 1)))) return st;
+        double* d_part = nullptr;
+        if ((st = tmp.alloc(&d_ne, (size_t)kBasis * (kBasis + 1))) ||
+            (st = tmp.alloc(&d_part, (size_t)kSetupBlocks * kNormalEntries)))
+            return st;
         LMOSEM_CK(c, cudaMemsetAsync(d_ne, 0, sizeof(double) * kBasis * (kBasis + 1), c->stream));
         LMOSEM_PROF_BEGIN(c);
-        k_basis_normal<<<dim3(kBasis, kBasis + 1), 256, 0, c->stream>>>(feat, targ, n, m, d_floor, d_ne);
+        k_basis_normal<<<kSetupBlocks, kSetupThreads, 0, c->stream>>>(feat, targ, n, m, d_floor, d_part);
+        LMOSEM_LAUNCHED(c, LMOSEM_K_SURROGATE);
+        LMOSEM_PROF_BEGIN(c);
+        k_basis_normal_sum<<<(kNormalEntries + 31) / 32, 32, 0, c->stream>>>(d_part, kSetupBlocks, d_ne);
         LMOSEM_LAUNCHED(c, LMOSEM_K_SURROGATE);
         double ne[kBasis * (kBasis + 1)];
         LMOSEM_CK(c, cudaMemcpyAsync(ne, d_ne, sizeof(ne), cudaMemcpyDeviceToHost, c->stream));
@@ -830,7 +945,7 @@ lmosem_status run_surrogate_train(lmosem_ctx* c, const float* feat, const float*
     float* d_floor = nullptr;
     int* d_step = nullptr;
     float* d_sc = nullptr;
-    double *d_cdf = nullptr, *d_csum = nullptr;
+    double *d_cdf = nullptr, *d_csum = nullptr, *d_sums = nullptr;
     float* tf = nullptr;  // (Scratch keeps the address of the pointer: same scope as tmp)
     Scratch tmp(c);
     if (rel && floor_below > 0.0f) {  // floor per event row: the targets floored once
@@ -851,7 +966,7 @@ lmosem_status run_surrogate_train(lmosem_ctx* c, const float* feat, const float*
         (st = tmp.alloc(&tb.grad, kParams)) ||
         (st = tmp.alloc(&tb.m, kParams)) || (st = tmp.alloc(&tb.v, kParams)) ||
         (st = tmp.alloc(&d_curve, std::max(1, steps))) || (st = tmp.alloc(&d_floor, 1)) ||
-        (st = tmp.alloc(&d_step, 1)) || (st = tmp.alloc(&d_sc, 3)))
+        (st = tmp.alloc(&d_step, 1)) || (st = tmp.alloc(&d_sc, 3)) || (st = tmp.alloc(&d_sums, 2 * kSetupBlocks)))
         return st;
     LMOSEM_CK(c, cudaMemsetAsync(tb.m, 0, sizeof(float) * kParams, c->stream));
     LMOSEM_CK(c, cudaMemsetAsync(tb.v, 0, sizeof(float) * kParams, c->stream));
@@ -861,7 +976,10 @@ lmosem_status run_surrogate_train(lmosem_ctx* c, const float* feat, const float*
     LMOSEM_LAUNCHED(c, LMOSEM_K_SURROGATE);
     if ((st = fit_baseline(c, feat, targ, n, d_floor, residual_fit, blob))) return st;
     LMOSEM_PROF_BEGIN(c);
-    k_target_stats<<<1, 256, 0, c->stream>>>(targ, feat, n, d_floor, blob);
+    k_target_sums<<<kSetupBlocks, kSetupThreads, 0, c->stream>>>(targ, feat, n, d_floor, blob, d_sums);
+    LMOSEM_LAUNCHED(c, LMOSEM_K_SURROGATE);
+    LMOSEM_PROF_BEGIN(c);
+    k_target_stats<<<1, 32, 0, c->stream>>>(d_sums, kSetupBlocks, n, blob);
     LMOSEM_LAUNCHED(c, LMOSEM_K_SURROGATE);
     const float b1 = 0.9f, b2 = 0.999f;
     // one training step: its scalars (minibatch index, loss slot, learning
@@ -877,10 +995,10 @@ lmosem_status run_surrogate_train(lmosem_ctx* c, const float* feat, const float*
         k_cdf_chunks<<<(unsigned)nchunks, 256, 0, c->stream>>>(rel, n, magnitude_power, d_csum);
         LMOSEM_LAUNCHED(c, LMOSEM_K_SURROGATE);
         LMOSEM_PROF_BEGIN(c);
-        k_cdf_offsets<<<1, 32, 0, c->stream>>>(d_csum, nchunks);
+        k_cdf_offsets<<<1, 1024, 0, c->stream>>>(d_csum, nchunks);
         LMOSEM_LAUNCHED(c, LMOSEM_K_SURROGATE);
         LMOSEM_PROF_BEGIN(c);
-        k_cdf_fill<<<(unsigned)nchunks, 32, 0, c->stream>>>(rel, n, magnitude_power, d_csum, d_cdf);
+        k_cdf_fill<<<(unsigned)nchunks, 256, 0, c->stream>>>(rel, n, magnitude_power, d_csum, d_cdf);
         LMOSEM_LAUNCHED(c, LMOSEM_K_SURROGATE);
     }
     tb.loss = d_curve;
