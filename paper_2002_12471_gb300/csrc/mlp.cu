@@ -120,6 +120,19 @@ __device__ __forceinline__ int64_t x_index(int64_t i, int k, bool tiled) {
     return (i >> 7) * (128 * kInPad) + (r >> 3) * 128 + (k >> 3) * 64 + (r & 7) * 8 + (k & 7);
 }
 
+// learning rate and Adam bias corrections of step s (the last 20% of the steps
+// at lr / 10): sc = (lr_s, 1 - b1^(s+1), 1 - b2^(s+1))
+struct StepScalars {
+    int steps;
+    float lr, b1, b2;
+    float* sc;
+};
+__device__ __forceinline__ void step_scalars(const StepScalars& S, int s) {
+    S.sc[0] = s < S.steps * 0.8 ? S.lr : S.lr * 0.1f;
+    S.sc[1] = (float)(1.0 - pow((double)S.b1, (double)(s + 1)));
+    S.sc[2] = (float)(1.0 - pow((double)S.b2, (double)(s + 1)));
+}
+
 // (step_ptr: the step index lives on the device, for a captured training step)
 // (cdf: inclusive prefix sums of sampling weights, n FP64 values: row i is
 // drawn with probability weight_i / total, by bisection; nullptr: uniform)
@@ -127,7 +140,13 @@ __global__ void k_gather(const float* __restrict__ feat, const float* __restrict
                          int B, uint64_t seed, int step, const int* __restrict__ step_ptr,
                          const double* __restrict__ cdf, const float* __restrict__ blob,
                          const float* __restrict__ floor, __nv_bfloat16* __restrict__ X, float* __restrict__ t,
-                         bool tiled) {
+                         bool tiled, StepScalars S) {
+    // one block more than the rows need forms the step's scalars beside them
+    // (9 us of the step's chain as a kernel of its own)
+    if (S.sc && blockIdx.x == gridDim.x - 1) {
+        if (threadIdx.x == 0) step_scalars(S, *step_ptr);
+        return;
+    }
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
     if (step_ptr) step = *step_ptr;
@@ -200,6 +219,7 @@ __global__ void __launch_bounds__(kH + 32) k_out_wgrad(const float* __restrict__
     const int per = (B + kOutSplits - 1) / kOutSplits;
     const int b0 = blockIdx.x * per, b1 = min(B, b0 + per);
     float s = 0.0f;
+#pragma unroll 16  // (loads in flight: 50 us with one at a time)
     for (int b = b0; b < b1; ++b) s += dy[b] * (k < kH ? __bfloat162float(H4[(int64_t)b * kH + k]) : 1.0f);
     part[blockIdx.x * (kH + 1) + k] = s;
 }
@@ -208,6 +228,7 @@ __global__ void k_out_wgrad_sum(const float* __restrict__ part, float* __restric
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k > kH) return;
     float s = 0.0f;
+#pragma unroll 16
     for (int z = 0; z < kOutSplits; ++z) s += part[z * (kH + 1) + k];
     grad[k < kH ? kOffW5 + k : kOffB5] = s;
 }
@@ -219,6 +240,7 @@ __global__ void k_rowsum(const __nv_bfloat16* __restrict__ ZT, int rows, int B, 
     const int lane = threadIdx.x & 31;
     if (r >= rows) return;
     float s = 0.0f;
+#pragma unroll 16
     for (int b = lane; b < B; b += 32) s += __bfloat162float(ZT[(int64_t)r * ld + b]);
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) out[r] = s;
@@ -231,18 +253,9 @@ __global__ void k_copy_grad(const float* __restrict__ src, int rows, int cols, i
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows * cols) return;
     float s = 0.0f;
+#pragma unroll 16
     for (int z = 0; z < splits; ++z) s += src[z * split_stride + (int64_t)(i / cols) * lds + (i % cols)];
     dst[i] = s;
-}
-
-// learning rate and Adam bias corrections of the step *step_ptr (the last
-// 20% of the steps at lr / 10): sc = (lr_s, 1 - b1^(s+1), 1 - b2^(s+1))
-__global__ void k_step_scalars(const int* __restrict__ step_ptr, int steps, float lr, float b1, float b2,
-                               float* __restrict__ sc) {
-    const int s = *step_ptr;
-    sc[0] = s < steps * 0.8 ? lr : lr * 0.1f;
-    sc[1] = (float)(1.0 - pow((double)b1, (double)(s + 1)));
-    sc[2] = (float)(1.0 - pow((double)b2, (double)(s + 1)));
 }
 
 // Adam (bias-corrected moments) over the whole blob except (mu, sigma); the
@@ -860,7 +873,7 @@ lmosem_status run_surrogate_grad(lmosem_ctx* c, const float* blob, const float* 
     if ((st = weights_bf16(c, blob, w))) return st;
     LMOSEM_PROF_BEGIN(c);
     k_gather<<<(B + 255) / 256, 256, 0, c->stream>>>(feat, targ, n, B, 0, 0, nullptr, nullptr, blob, nullptr, tb.X,
-                                                     tb.t, false);
+                                                     tb.t, false, StepScalars{});
     LMOSEM_LAUNCHED(c, LMOSEM_K_SURROGATE);
     tb.grad = grad_out;
     if ((st = loss_grad(c, blob, w, tb, B))) return st;
@@ -1007,13 +1020,11 @@ lmosem_status run_surrogate_train(lmosem_ctx* c, const float* feat, const float*
         lmosem_status s2;
         if ((s2 = weights_bf16(c, blob, w))) return s2;
         LMOSEM_PROF_BEGIN(c);
-        k_gather<<<(B + 255) / 256, 256, 0, c->stream>>>(feat, targ, n, B, seed | 1ull, 0, d_step, d_cdf, blob,
-                                                         d_floor, tb.X, tb.t, false);
+        k_gather<<<(B + 255) / 256 + 1, 256, 0, c->stream>>>(feat, targ, n, B, seed | 1ull, 0, d_step, d_cdf, blob,
+                                                             d_floor, tb.X, tb.t, false,
+                                                             StepScalars{steps, lr, b1, b2, d_sc});
         LMOSEM_LAUNCHED(c, LMOSEM_K_SURROGATE);
         if ((s2 = loss_grad(c, blob, w, tb, B))) return s2;
-        LMOSEM_PROF_BEGIN(c);
-        k_step_scalars<<<1, 1, 0, c->stream>>>(d_step, steps, lr, b1, b2, d_sc);
-        LMOSEM_LAUNCHED(c, LMOSEM_K_SURROGATE);
         LMOSEM_PROF_BEGIN(c);
         k_adam<<<(unsigned)((kOffBase + 255) / 256), 256, 0, c->stream>>>(blob, tb.grad, tb.m, tb.v, kOffBase, d_sc, b1,
                                                                        b2, 1e-8f, d_step);
@@ -1073,7 +1084,7 @@ lmosem_status run_surrogate_infer(lmosem_ctx* c, const float* blob, const float*
     if ((st = infer_weights(c, blob, w, tmp))) return st;
     LMOSEM_PROF_BEGIN(c);
     k_gather<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(feat, feat, n, (int)n, 0, 0, nullptr, nullptr, blob, nullptr, X, out,
-                                                                 c->surrogate_kernel != 1);
+                                                                 c->surrogate_kernel != 1, StepScalars{});
     LMOSEM_LAUNCHED(c, LMOSEM_K_SURROGATE);
     __nv_bfloat16* Hs[4] = {H, H + n * kH, H + 2 * n * kH, H + 3 * n * kH};
     if ((st = forward_infer(c, blob, w, X, Hs, out, n))) return st;

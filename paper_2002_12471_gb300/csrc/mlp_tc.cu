@@ -574,23 +574,51 @@ __global__ void __launch_bounds__(128) k_gemm_tc(GemmTcArgs G) {
             if (gr >= G.M) continue;
             const int col0 = n0 + c0;
             const int nv = min(32, G.N - col0);
+            // A thread owns 32 consecutive columns of a row: 16-byte loads and
+            // stores of 8 BF16 or 4 FP32 values (rows and column groups are
+            // 16-byte aligned: ldc and ldm are multiples of 8), single ones in a
+            // ragged last group.  With single 2-byte accesses the 8,192 x 256 x
+            // 256 products took 33 (bias) and 45 us (mask).
             if constexpr (EPI == 0) {
                 float* out = reinterpret_cast<float*>(G.C) + (int64_t)blockIdx.z * G.split_stride + gr * G.ldc + col0;
 #pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    if (j < nv) out[j] = __uint_as_float(r[j]);
+                for (int j = 0; j < 32; j += 4) {
+                    if (j + 4 <= nv) {
+                        *reinterpret_cast<uint4*>(out + j) = make_uint4(r[j], r[j + 1], r[j + 2], r[j + 3]);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (j + i < nv) out[j + i] = __uint_as_float(r[j + i]);
+                    }
+                }
             } else {
                 __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(G.C) + gr * G.ldc + col0;
+                const __nv_bfloat16* mk = EPI == 2 ? G.mask + gr * G.ldm + col0 : nullptr;
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    if (j >= nv) continue;
-                    float v = __uint_as_float(r[j]);
-                    if constexpr (EPI == 1) {
-                        v = fmaxf(v + G.bias[col0 + j], 0.0f);
+                for (int j = 0; j < 32; j += 8) {
+                    if (j + 8 <= nv) {
+                        uint4 m4 = make_uint4(0u, 0u, 0u, 0u), o4;
+                        if constexpr (EPI == 2) m4 = *reinterpret_cast<const uint4*>(mk + j);
+                        const __nv_bfloat16* m8 = reinterpret_cast<const __nv_bfloat16*>(&m4);
+                        __nv_bfloat16* o8 = reinterpret_cast<__nv_bfloat16*>(&o4);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            float v = __uint_as_float(r[j + i]);
+                            if constexpr (EPI == 1) v = fmaxf(v + G.bias[col0 + j + i], 0.0f);
+                            else v = __bfloat162float(m8[i]) > 0.0f ? v : 0.0f;
+                            o8[i] = __float2bfloat16_rn(v);
+                        }
+                        *reinterpret_cast<uint4*>(out + j) = o4;
                     } else {
-                        v = __bfloat162float(G.mask[gr * G.ldm + col0 + j]) > 0.0f ? v : 0.0f;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            if (j + i >= nv) continue;
+                            float v = __uint_as_float(r[j + i]);
+                            if constexpr (EPI == 1) v = fmaxf(v + G.bias[col0 + j + i], 0.0f);
+                            else v = __bfloat162float(mk[j + i]) > 0.0f ? v : 0.0f;
+                            out[j + i] = __float2bfloat16_rn(v);
+                        }
                     }
-                    out[j] = __float2bfloat16_rn(v);
                 }
             }
         }
