@@ -11,7 +11,7 @@
 // Gaussians and to interpolate it at every event than to form the sum per
 // event.  The grid is uniform in u (step at most 0.415 of the narrowest sigma_u)
 // and in x = 2 sqrt(E / kappa) (sigma_E^2 = kappa E, so every Gaussian has unit
-// width in x; step 0.22), with 12 x 8 point stencils.
+// width in x; step 0.25), with 12 x 8 point stencils.
 //
 // On the grid the sum is a matrix product per angle and energy node,
 //     T[k][i][n] = sum_m U[i][m] G_k[n][m],  G_k = W phi(E_k; E', sigma_E),
@@ -46,6 +46,7 @@ constexpr uint32_t kColMain = 0, kColPart = 2 * kWin, kColA = 4 * kWin;
 static_assert(kColA + kASlots * 16 == 512, "tensor memory columns");
 constexpr int kGenWarps = 16, kEpiWarps = 8, kMmaWarp = 24, kLoadWarp = 25, kGridThreads = 26 * 32;
 constexpr int kEpi = 16;                     // columns per step of the epilogue
+static_assert(kSub == 64, "two ballots");
 static_assert(kEpi == 16 && kWin % kEpi == 0 && kWin % 16 == 0, "whole steps");
 constexpr int kEGroup = 8;                  // energy nodes per CTA: 4 lane groups x 2
 constexpr int kNTile = 32;                  // support pixels per CTA
@@ -85,18 +86,23 @@ __global__ void k_grid_groups(const float4* __restrict__ mpar, const int32_t* __
     for (int r = threadIdx.x; r < n_scat; r += blockDim.x) su[r] = mpar[(size_t)a * n_scat + o[r]].x;
     for (int r = threadIdx.x; r < max_sub * kSub; r += blockDim.x) slot_m[(size_t)a * max_sub * kSub + r] = -1;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {  // one warp walks the starts, testing kSub = 64 pixels at a time
+        const int lane = threadIdx.x;
         int g = 0;
         for (int r = 0; r < n_scat && g < max_sub; ++g) {
-            start[g] = r;
+            if (lane == 0) start[g] = r;
             const float lim = su[r] + span;
-            const int e = min(n_scat, r + kSub);
-            while (r < e && su[r] <= lim) ++r;
+            const unsigned b0 = __ballot_sync(0xffffffffu, r + lane < n_scat && su[min(r + lane, n_scat - 1)] <= lim);
+            const unsigned b1 =
+                __ballot_sync(0xffffffffu, r + 32 + lane < n_scat && su[min(r + 32 + lane, n_scat - 1)] <= lim);
+            r += __popc(b0) + __popc(b1);  // sorted: the positions within the span are the first ones
         }
-        start[g] = n_scat;
-        ns = g;
-        n_sub[a] = g;
-        urange[a] = make_float2(su[0], su[n_scat - 1]);
+        if (lane == 0) {
+            start[g] = n_scat;
+            ns = g;
+            n_sub[a] = g;
+            urange[a] = make_float2(su[0], su[n_scat - 1]);
+        }
     }
     __syncthreads();
     for (int g = threadIdx.x; g < ns; g += blockDim.x) {
@@ -420,8 +426,9 @@ constexpr uint32_t kSmBytes = kSmMisc + 16;
 // (a subgroup), which reach the kWin nodes from i0 on: so the columns of the
 // accumulators are a ring of kWin nodes that slides along u, a node's value
 // being complete (and stored) once i0 has passed it.
-//  * 8 generator warps form G of a chunk (16 scatter pixels) for both energy
-//    nodes of their lanes and write its FP16 parts to tensor memory;
+//  * 16 generator warps (4 lane quarters x 4 chunks of 16 scatter pixels) form
+//    G of their chunk for both energy nodes of their quarter and write its FP16
+//    parts to tensor memory;
 //  * the load warp brings U by bulk copies;
 //  * the MMA warp sums the 4 chunks of a subgroup into a partial accumulator
 //    (3 products per chunk: low x high, high x low, high x high);
@@ -429,6 +436,15 @@ constexpr uint32_t kSmBytes = kSmMisc + 16;
 //    the tensor core truncates its running sum (measured: -8e-8 relative per
 //    product of a growing sum, -5e-6 after 64), so chains are kept to one
 //    subgroup and the long sum is rounded to nearest.
+// What bounds it: issue.  A subgroup takes 2,280 cycles per CTA at 128 x 128,
+// of which its 24 products need 1,152 on the tensor cores; the generators' and
+// the epilogue's 1,590 instructions per scheduler (exponentials, FP16 splits,
+// tensor-memory loads, FP32 adds) keep the schedulers 65-70% busy, and the
+// hand-over of a chunk between the roles takes the rest.  Measured at 128 x
+// 128: three products of N = 112 take 213 cycles when lane 0 issues them, 168
+// with elect.sync; plane values by __ldg made a subgroup 3,450 to 5,600 cycles,
+// by bulk copies 2,700; a slot of A for every chunk and node and windows of 96
+// nodes took an angle from 1.10 to 0.98 ms; two issuing warps 1.00.
 __global__ void __launch_bounds__(kGridThreads, 1) k_grid_sum(SumArgs A) {
     extern __shared__ __align__(1024) unsigned char sm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -742,25 +758,29 @@ struct CellArgs {
     float e_min, e_max;
     double u_lo, inv_hu, x_lo, inv_hx, inv_kappa;
     int nce, ncu, n_slots;
+    int nbx, nbu;          // blocks of 2 x 2 cells
 };
-// cell of an event; events outside the grid's region: n_slots nce ncu + slot
-__device__ __forceinline__ int grid_cell(const CellArgs& A, int64_t r, double* fu, double* fx) {
+// block of 2 x 2 cells of an event (*sub: its cell, 2 in x + in u); events
+// outside the grid's region: n_slots nbx nbu + slot
+__device__ __forceinline__ int grid_block(const CellArgs& A, int64_t r, double* fu, double* fx, int* sub) {
     const int a = A.a_s[r], s = A.angle_slot[a];
     const float u = A.u_s[r], e = A.e_s[r];
     const float2 ur = A.urange[a];
-    const int out = A.n_slots * A.nce * A.ncu + s;
+    const int out = A.n_slots * A.nbx * A.nbu + s;
     if (!(u >= ur.x - A.edge && u <= ur.y + A.edge && e >= A.e_min && e <= A.e_max)) return out;
     const double pu = ((double)u - A.u_lo) * A.inv_hu, px = (2.0 * sqrt((double)e * A.inv_kappa) - A.x_lo) * A.inv_hx;
     const int cu = (int)floor(pu), cx = (int)floor(px);
     if (cu < 0 || cu >= A.ncu || cx < 0 || cx >= A.nce) return out;
     *fu = pu - cu;
     *fx = px - cx;
-    return (s * A.nce + cx) * A.ncu + cu;
+    *sub = 2 * (cx & 1) + (cu & 1);
+    return (s * A.nbx + (cx >> 1)) * A.nbu + (cu >> 1);
 }
 __global__ void k_grid_count(CellArgs A, int32_t* __restrict__ cnt) {
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     double fu, fx;
-    if (r < A.J) atomicAdd(cnt + grid_cell(A, r, &fu, &fx), 1);
+    int sub;
+    if (r < A.J) atomicAdd(cnt + grid_block(A, r, &fu, &fx, &sub), 1);
 }
 // events of the input outside the grid's region (before the sort)
 __global__ void k_grid_outside(CellArgs A, int32_t* __restrict__ n) {
@@ -770,14 +790,16 @@ __global__ void k_grid_outside(CellArgs A, int32_t* __restrict__ n) {
         const int a = A.a_s[r];
         if (a >= 0 && a < A.n_slots) {
             double fu, fx;
-            out = grid_cell(A, r, &fu, &fx) >= A.n_slots * A.nce * A.ncu;
+            int sub;
+            out = grid_block(A, r, &fu, &fx, &sub) >= A.n_slots * A.nbx * A.nbu;
         }
     }
     const unsigned b = __ballot_sync(0xffffffffu, out);
     if (b && (threadIdx.x & 31) == 0) atomicAdd(n, __popc(b));
 }
 
-// an event in cell order: its row, cell, position and energy, and its weights
+// an event in block order: its row, cell (4 x block + cell of the block; outside
+// the grid the key itself), position and energy, and its weights
 struct __align__(16) GridEvent {
     int32_t row, cell;
     float u, e;
@@ -790,23 +812,24 @@ __global__ void k_grid_place(CellArgs A, Stencil<kPU> su, Stencil<kPE> sx, const
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= A.J) return;
     double fu = 0.0, fx = 0.0;
-    const int c = grid_cell(A, r, &fu, &fx);
+    int sub = 0;
+    const int c = grid_block(A, r, &fu, &fx, &sub);
     GridEvent ev;
     ev.row = (int32_t)r;
-    ev.cell = c;
+    ev.cell = c < A.n_slots * A.nbx * A.nbu ? 4 * c + sub : c;
     ev.u = A.u_s[r];
     ev.e = A.e_s[r];
     stencil_weights<kPU>(su, fu, ev.wu);
     stencil_weights<kPE>(sx, fx, ev.we);
-    // the order inside a cell does not matter: every row is formed by itself
+    // the order inside a block does not matter: every row is formed by itself
     out[off[c] + atomicAdd(fill + c, 1)] = ev;
 }
 
 struct RowArgs {
     const GridEvent* ev;
-    const int32_t* off;          // first event of every cell
-    int cell0, cell1;            // cells of the group
-    int nce, ncu, ne, nu, s0;
+    const int32_t* off;          // first event of every block
+    int cell0, cell1;            // blocks of the group
+    int nbx, nbu, ne, nu, s0;
     const int32_t* slot_angle;
     const float* T;
     int n_sup, ld;
@@ -817,9 +840,28 @@ struct RowArgs {
     int64_t ld_out, row_base;
 };
 
-// Rows of 64 events (in cell order) x 128 support pixels: the 12 x 8 grid
-// values around a cell are loaded once for all of the cell's events.
+// Rows of 64 events (in block order) x 128 support pixels: the 13 x 9 grid
+// values around a block of 2 x 2 cells are loaded once for all of its events.
+// The loads bound the kernel (one L1 wavefront per value and warp): blocks of
+// 2 x 2 cells hold about twice the events of a cell for 1.2 times the values
+// (per 33k events x 5,884 pixels 1.97 -> 1.78 ms).  Slower: moving the values
+// of a neighbouring block up in registers (2.20 ms, 186 registers) and
+// prefetching the next block's lines to L1 (2.25 ms).
 constexpr int kRowEvents = 64;
+template <int OX, int OU>
+__device__ __forceinline__ float stencil_sum(const float (&tv)[kPE + 1][kPU + 1], const float (&we)[kPE],
+                                             const float (&wu)[kPU]) {
+    float acc = 0.0f;
+#pragma unroll
+    for (int q = 0; q < kPE; ++q) {
+        float2 v = make_float2(0.0f, 0.0f);
+#pragma unroll
+        for (int k = 0; k < kPU; k += 2)
+            v = fma2(make_float2(wu[k], wu[k + 1]), make_float2(tv[q + OX][k + OU], tv[q + OX][k + OU + 1]), v);
+        acc = fmaf(we[q], v.x + v.y, acc);
+    }
+    return acc;
+}
 __global__ void __launch_bounds__(128) k_grid_rows(RowArgs A) {
     __shared__ float4 sev[kRowEvents * 6];
     const int p0 = A.off[A.cell0] + blockIdx.x * kRowEvents, p1 = min(A.off[A.cell1], p0 + kRowEvents);
@@ -830,44 +872,39 @@ __global__ void __launch_bounds__(128) k_grid_rows(RowArgs A) {
     const int n = blockIdx.y * 128 + threadIdx.x;
     if (n >= A.ld) return;
     const bool real = n < A.n_sup;
-    float tv[kPE][kPU];
+    float tv[kPE + 1][kPU + 1];
     float4 pp = make_float4(0.0f, 0.0f, -INFINITY, 0.0f);
-    int cell = -1;
+    int block = -1;
     for (int p = 0; p < p1 - p0; ++p) {
         const float4 h = sev[p * 6];
         const int row = __float_as_int(h.x), c = __float_as_int(h.y);
-        if (c != cell) {
-            cell = c;
-            const int cu = c % A.ncu, cx = (c / A.ncu) % A.nce, s = c / (A.ncu * A.nce);
+        if ((c >> 2) != block) {
+            block = c >> 2;
+            const int cu = 2 * (block % A.nbu), cx = 2 * ((block / A.nbu) % A.nbx), s = block / (A.nbu * A.nbx);
             const float* t = A.T + ((((size_t)(s - A.s0) * gridDim.y + blockIdx.y) * A.ne + cx) * A.nu + cu) * kTCols +
                              threadIdx.x;
 #pragma unroll
-            for (int q = 0; q < kPE; ++q) {
+            for (int q = 0; q <= kPE; ++q) {
+                if (q == kPE && cx + q >= A.ne) break;  // the last block may hold one row of cells only
 #pragma unroll
-                for (int k = 0; k < kPU; ++k) tv[q][k] = __ldg(t + k * kTCols);
+                for (int k = 0; k <= kPU; ++k) tv[q][k] = __ldg(t + k * kTCols);
                 t += (size_t)A.nu * kTCols;
             }
             if (real) pp = __ldg(A.ppar + (size_t)A.slot_angle[s] * A.ld_w + n);
         }
-        const float* we = reinterpret_cast<const float*>(sev + p * 6 + 1);
-        float wu[kPU];
+        float we[kPE], wu[kPU];
 #pragma unroll
-        for (int k = 0; k < kPU / 4; ++k) {
-            const float4 v = sev[p * 6 + 3 + k];
-            wu[4 * k] = v.x;
-            wu[4 * k + 1] = v.y;
-            wu[4 * k + 2] = v.z;
-            wu[4 * k + 3] = v.w;
+        for (int k = 0; k < (kPE + kPU) / 4; ++k) {
+            const float4 v = sev[p * 6 + 1 + k];
+            float* w = k < kPE / 4 ? we + 4 * k : wu + 4 * (k - kPE / 4);
+            w[0] = v.x;
+            w[1] = v.y;
+            w[2] = v.z;
+            w[3] = v.w;
         }
-        float acc = 0.0f;
-#pragma unroll
-        for (int q = 0; q < kPE; ++q) {
-            float2 v = make_float2(0.0f, 0.0f);
-#pragma unroll
-            for (int k = 0; k < kPU; k += 2)
-                v = fma2(make_float2(wu[k], wu[k + 1]), make_float2(tv[q][k], tv[q][k + 1]), v);
-            acc = fmaf(we[q], v.x + v.y, acc);
-        }
+        float acc;
+        if (c & 2) acc = (c & 1) ? stencil_sum<1, 1>(tv, we, wu) : stencil_sum<1, 0>(tv, we, wu);
+        else acc = (c & 1) ? stencil_sum<0, 1>(tv, we, wu) : stencil_sum<0, 0>(tv, we, wu);
         const float te = (h.w - A.e0) * A.sE0, tu = (h.z - pp.x) * pp.y;
         const float prim = ex2_approx(fmaf(-tu, tu, pp.z + fmaf(-te, te, A.lE0)));
         // the sum is never negative; an interpolated zero may be, by its rounding
@@ -951,6 +988,8 @@ CellArgs cell_args(const lmosem_ctx* c, const int32_t* a, const float* u, const 
     A.nce = G.nce;
     A.ncu = G.ncu;
     A.n_slots = c->n_angles;
+    A.nbx = (G.nce + 1) / 2;
+    A.nbu = (G.ncu + 1) / 2;
     return A;
 }
 
@@ -1001,7 +1040,7 @@ lmosem_status grid_plan(lmosem_ctx* c, int64_t n, bool* use) {
         const double ext = std::min(half, rmax + G.edge);
         G.u_lo = -ext;
         G.ncu = (int)floor(2.0 * ext / G.hu) + 1;
-        G.nu = G.ncu + kPU - 1;
+        G.nu = (G.ncu + 1) / 2 * 2 + kPU - 1;  // whole blocks of 2 cells
         const double kappa = kappa_of(c), e_min = c->e0 / (1.0 + 2.0 * c->e0 / kMec2Kev);
         G.e_min = std::max(c->e_lo, e_min - 1.5 * sqrt(kappa * e_min));
         G.e_max = std::min(c->e_hi, c->e0 + kEdgeSigma * sqrt(kappa * c->e0));
@@ -1019,47 +1058,52 @@ lmosem_status grid_plan(lmosem_ctx* c, int64_t n, bool* use) {
         G.log_u = (float)(14 - (int)ceil(log2(ub)));
         if (!(fabs(G.log_g) < 60.0f && fabs(G.log_u) < 30.0f)) return LMOSEM_OK;
 
-        lmosem_status st;
-        const size_t na = c->n_angles;
-        int32_t* order = nullptr;
-        Scratch tmp(c);
-        if ((st = tmp.alloc(&order, na * c->n_scat)) || (st = dev_alloc(c, &G.d_slot_m, na * G.max_sub * kSub)) ||
-            (st = dev_alloc(c, &G.d_i0, na * G.max_sub)) || (st = dev_alloc(c, &G.d_n_sub, na)) ||
-            (st = dev_alloc(c, &G.d_urange, na)) || (st = dev_alloc(c, &G.d_enode, G.ne / 2)) ||
-            (st = dev_alloc(c, &G.d_angle_slot, na)))
-            return st;
-        std::vector<float4> en(G.ne / 2);
-        const double cE2 = (float)(1.4426950408889634 / (2.0 * kappa));  // as the tables' FP32 factor
-        auto node = [&](int k) {
-            const double x = G.x_lo + (k - (kPE / 2 - 1)) * kRhoX;
-            return cE2 * kappa * 0.25 * x * x;
-        };
-        for (int k = 0; k < G.ne / 2; ++k) {
-            const double e0 = node(2 * k);
-            const float hi = (float)e0;
-            en[k] = make_float4(hi, (float)(e0 - hi), (float)(node(2 * k + 1) - e0), 0.0f);
-        }
-        LMOSEM_CK(c, cudaMemcpyAsync(G.d_enode, en.data(), en.size() * sizeof(float4), cudaMemcpyHostToDevice, c->stream));
-        LMOSEM_PROF_BEGIN(c);
-        k_grid_rank<<<dim3((c->n_scat + 255) / 256, c->n_angles), 256, 0, c->stream>>>(c->d_mpar, c->n_scat, order);
-        LMOSEM_LAUNCHED(c, LMOSEM_K_TABLES);
-        const size_t smem = sizeof(float) * ((size_t)c->n_scat + G.max_sub + 1);
-        LMOSEM_CK(c, cudaFuncSetAttribute(k_grid_groups, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        LMOSEM_PROF_BEGIN(c);
-        k_grid_groups<<<c->n_angles, 256, smem, c->stream>>>(
-            c->d_mpar, order, c->n_scat, G.max_sub, (float)span, (float)cut,
-            (float)(G.u_lo - (kPU / 2 - 1) * G.hu), (float)(1.0 / G.hu), G.d_slot_m, G.d_i0, G.d_n_sub, G.d_urange);
-        LMOSEM_LAUNCHED(c, LMOSEM_K_TABLES);
+        G.span = span;
         G.n_sub = 1 + (int)(1.1 * std::max((double)c->n_scat / kSub, 2.0 * rmax / span));
         G.strip = std::min(1.0, 1.2 * c->k_sigma * s_lat / rmax);
-        G.state = 2;
+        G.state = 2;  // parameters known, tables not made
     }
-    if (G.state != 2) return LMOSEM_OK;
+    if (G.state < 2) return LMOSEM_OK;
     const double per_s = 152.0 * 1.92e9, tiles = (c->n_sup + 127) / 128;
     const double t_grid = c->n_angles * ((c->n_sup + kNTile - 1) / kNTile * (G.ne / kEGroup) * (2300.0 * G.n_sub + 9000.0) / per_s +
                                          tiles * G.n_sub * 25e-9) + n * tiles * 400.0 / per_s + 60e-6;
     const double t_path = n * (0.8 * G.strip * c->n_scat * c->n_sup) / 5.5e12;
-    *use = t_grid < 0.9 * t_path;
+    if (!(t_grid < 0.9 * t_path)) return LMOSEM_OK;
+    *use = true;
+    if (G.state == 3) return LMOSEM_OK;
+    const double kappa = kappa_of(c);
+    lmosem_status st;
+    const size_t na = c->n_angles;
+    int32_t* order = nullptr;
+    Scratch tmp(c);
+    if ((st = tmp.alloc(&order, na * c->n_scat)) || (st = dev_alloc(c, &G.d_slot_m, na * G.max_sub * kSub)) ||
+        (st = dev_alloc(c, &G.d_i0, na * G.max_sub)) || (st = dev_alloc(c, &G.d_n_sub, na)) ||
+        (st = dev_alloc(c, &G.d_urange, na)) || (st = dev_alloc(c, &G.d_enode, G.ne / 2)) ||
+        (st = dev_alloc(c, &G.d_angle_slot, na)))
+        return st;
+    std::vector<float4> en(G.ne / 2);
+    const double cE2 = (float)(1.4426950408889634 / (2.0 * kappa));  // as the tables' FP32 factor
+    auto node = [&](int k) {
+        const double x = G.x_lo + (k - (kPE / 2 - 1)) * kRhoX;
+        return cE2 * kappa * 0.25 * x * x;
+    };
+    for (int k = 0; k < G.ne / 2; ++k) {
+        const double e0 = node(2 * k);
+        const float hi = (float)e0;
+        en[k] = make_float4(hi, (float)(e0 - hi), (float)(node(2 * k + 1) - e0), 0.0f);
+    }
+    LMOSEM_CK(c, cudaMemcpyAsync(G.d_enode, en.data(), en.size() * sizeof(float4), cudaMemcpyHostToDevice, c->stream));
+    LMOSEM_PROF_BEGIN(c);
+    k_grid_rank<<<dim3((c->n_scat + 255) / 256, c->n_angles), 256, 0, c->stream>>>(c->d_mpar, c->n_scat, order);
+    LMOSEM_LAUNCHED(c, LMOSEM_K_TABLES);
+    const size_t smem = sizeof(float) * ((size_t)c->n_scat + G.max_sub + 1);
+    LMOSEM_CK(c, cudaFuncSetAttribute(k_grid_groups, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LMOSEM_PROF_BEGIN(c);
+    k_grid_groups<<<c->n_angles, 256, smem, c->stream>>>(
+        c->d_mpar, order, c->n_scat, G.max_sub, (float)G.span, (float)G.cut,
+        (float)(G.u_lo - (kPU / 2 - 1) * G.hu), (float)(1.0 / G.hu), G.d_slot_m, G.d_i0, G.d_n_sub, G.d_urange);
+    LMOSEM_LAUNCHED(c, LMOSEM_K_TABLES);
+    G.state = 3;
     return LMOSEM_OK;
 }
 
@@ -1096,7 +1140,8 @@ lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& s
     const int ns = (int)slot_angle.size(), ld = (int)c->ld_model;
     const int64_t J = c->J;
     const double kappa = kappa_of(c), se0 = sqrt(kappa * c->e0);
-    const int64_t ncells = (int64_t)ns * G.nce * G.ncu, nkeys = ncells + ns;
+    const int nbx = (G.nce + 1) / 2, nbu = (G.ncu + 1) / 2;
+    const int64_t ncells = (int64_t)ns * nbx * nbu, nkeys = ncells + ns;
 
     // ---- events in cell order, with their weights
     std::vector<int32_t> slots(2 * ns);
@@ -1129,7 +1174,10 @@ lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& s
     const int64_t pairs = (int64_t)G.max_sub * kSub / 2;
     const int64_t plane_n = pairs * ld, t_n = (int64_t)G.ne * G.nu * ((ld + kTCols - 1) / kTCols * kTCols), u_n = (int64_t)G.max_sub * kUStage;
     const int64_t per_angle = plane_n * 16 + t_n * 4 + u_n;
-    const int gsz = (int)std::max<int64_t>(1, std::min<int64_t>(ns, c->table_budget / per_angle));
+    // groups of at most 2 GiB: the pool maps fresh memory at about 0.7 ms per GB (64 x 64 with 200k events: build
+    // 17.3 ms at 2 GiB, 18.2 at 1 GiB, 19.1 at 4 GiB)
+    const int gsz = (int)std::max<int64_t>(
+        1, std::min<int64_t>(ns, std::min<int64_t>(c->table_budget, int64_t(2) << 30) / per_angle));
     float4* planes = nullptr;
     float* T = nullptr;
     unsigned char* ublob = nullptr;
@@ -1230,10 +1278,10 @@ lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& s
         RowArgs R;
         R.ev = ev;
         R.off = off;
-        R.cell0 = s0 * G.nce * G.ncu;
-        R.cell1 = (s0 + na) * G.nce * G.ncu;
-        R.nce = G.nce;
-        R.ncu = G.ncu;
+        R.cell0 = s0 * nbx * nbu;
+        R.cell1 = (s0 + na) * nbx * nbu;
+        R.nbx = nbx;
+        R.nbu = nbu;
         R.ne = G.ne;
         R.nu = G.nu;
         R.s0 = s0;

@@ -30,9 +30,9 @@ constexpr int kBuildThreads = 256;
 // Grid of the scatter sum (grid.cu): its nodes, and per angle the scatter
 // pixels in subgroups of neighbouring positions.
 struct GridPlan {
-    int state = 0;               // 0: not made, 1: not usable for this problem, 2: ready
+    int state = 0;               // 0: not made, 1: not usable for this problem, 2: parameters, 3: tables
     double hu = 0, rho_u = 0;    // step in u; in units of the interpolation kernel's width
-    double cut = 0;              // longest position cut (mm)
+    double cut = 0, span = 0;    // longest position cut and subgroup (mm)
     double u_lo = 0, x_lo = 0;   // first cell edge in u and in x = 2 sqrt(E / kappa)
     int ncu = 0, nce = 0;        // cells
     int nu = 0, ne = 0;          // nodes

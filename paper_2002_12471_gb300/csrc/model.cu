@@ -1183,8 +1183,12 @@ lmosem_status build_model_rows(lmosem_ctx* c) {
     const int ns = (int)slot_angle.size();
     if (c->use_grid && !c->scatter_only) {
         dev_free(c, &c->d_wtab_all);  // the grid has tables of its own
-        c->terms_valid = c->terms_pending = true;
-        return build_model_rows_grid(c, slot_angle);
+        st = build_model_rows_grid(c, slot_angle);
+        if (st != LMOSEM_ENOMEM) {
+            c->terms_valid = c->terms_pending = st == LMOSEM_OK;
+            return st;
+        }
+        c->use_grid = false;  // its buffers do not fit beside the model: path by path
     }
     c->terms_pending = false;
 

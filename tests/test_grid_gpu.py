@@ -10,16 +10,14 @@ import numpy as np
 import pytest
 
 import oracle
-from _helpers import gpu_reconstruct, oracle_problem
+from tests._helpers import gpu_reconstruct, oracle_problem
 from paper_2002_12471_gb300 import synthetic as S
 
 pytestmark = pytest.mark.gpu
 
 
-def _case(n, angles, per_angle, seed, mu=None):
+def _case(n, angles, per_angle, seed):
     ph = S.brain_phantom(n, 256.0 / n)
-    if mu is not None:
-        ph.mu = mu(ph.mu)
     g = S.geometry(angles, n, 256.0 / n, 150.0, angle0_rad=0.2)
     ev = S.simulate_events(ph, g, angles * per_angle, seed=seed, batch=1 << 18)
     half = 0.5 * n * ph.pixel_mm
