@@ -833,29 +833,67 @@ __global__ void __launch_bounds__(kBuildThreads, 2) k_pathsum(PathSumArgs A) {
 // maximum in the normal range; 1 for BF16).  The scale cancels in the EM
 // update (paper Eq. 8: y_j and p_jq scale together) and enters only the
 // log-likelihood.
-template <typename H>
-__global__ void k_quantize(const float* __restrict__ stage, int64_t ld_stage, int64_t rows,
-                           int n_cols, int64_t ld_out, H* __restrict__ out, int64_t row0,
-                           float* __restrict__ scale, float hmax) {
-    int warps = blockDim.x >> 5;
-    int64_t r = (int64_t)blockIdx.x * warps + (threadIdx.x >> 5);
-    int lane = threadIdx.x & 31;
-    if (r >= rows) return;
-    const float* src = stage + r * ld_stage;
+// A CTA holds a row in registers between the search for its maximum and the
+// rounding, so that it is read once: with a warp per row the rows in flight
+// (152 SMs x 64 warps x 24 KB at 128 x 128) did not fit L2 and came from HBM
+// twice.  Rows wider than kQuantVec vectors per thread are read again.
+// NT = 64 up to 2,048 columns, where 256 threads held two loads each.
+constexpr int kQuantVec = 8;
+template <typename H, int NT>
+__global__ void __launch_bounds__(NT) k_quantize(const float* __restrict__ stage, int64_t ld_stage,
+                                                            int n_cols, int64_t ld_out, H* __restrict__ out,
+                                                            int64_t row0, float* __restrict__ scale, float hmax) {
+    __shared__ float smax[NT / 32];
+    const int64_t r = blockIdx.x;
+    const int t = threadIdx.x, nvec = (int)(ld_out / 4);  // ld_out and ld_stage are multiples of 32
+    const float4* src = reinterpret_cast<const float4*>(stage + r * ld_stage);
+    auto load = [&](int k) {  // columns beyond the support count as zero
+        float4 v = __ldcs(src + k);
+        if (4 * k + 3 >= n_cols) {
+            if (4 * k >= n_cols) v.x = 0.0f;
+            if (4 * k + 1 >= n_cols) v.y = 0.0f;
+            if (4 * k + 2 >= n_cols) v.z = 0.0f;
+            v.w = 0.0f;
+        }
+        return v;
+    };
+    float4 v[kQuantVec];
     float mx = 0.0f;
-    for (int n = lane; n < n_cols; n += 32) mx = fmaxf(mx, src[n]);
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    float c = mx > 0.0f ? mx / hmax : 1.0f;
-    float ic = 1.0f / c;
-    H* dst = out + (row0 + r) * ld_out;
-    for (int n = lane; n < ld_out; n += 32) {
-        float v = n < n_cols ? src[n] * ic : 0.0f;
-        if constexpr (std::is_same<H, __half>::value)
-            dst[n] = __float2half_rn(v);
-        else
-            dst[n] = __float2bfloat16_rn(v);
+#pragma unroll
+    for (int i = 0; i < kQuantVec; ++i) {
+        const int k = t + i * NT;
+        v[i] = k < nvec ? load(k) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        mx = fmaxf(fmaxf(fmaxf(mx, v[i].x), fmaxf(v[i].y, v[i].z)), v[i].w);
     }
-    if (lane == 0) scale[row0 + r] = c;
+    for (int k = t + kQuantVec * NT; k < nvec; k += NT) {
+        const float4 w = load(k);
+        mx = fmaxf(fmaxf(fmaxf(mx, w.x), fmaxf(w.y, w.z)), w.w);
+    }
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((t & 31) == 0) smax[t >> 5] = mx;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) mx = fmaxf(mx, smax[w]);
+    const float c = mx > 0.0f ? mx / hmax : 1.0f;
+    const float ic = 1.0f / c;
+    H* dst = out + (row0 + r) * ld_out;
+    auto store = [&](int k, float4 w) {
+        uint2 p;
+        if constexpr (std::is_same<H, __half>::value) {
+            const __half2 a = __floats2half2_rn(w.x * ic, w.y * ic), b = __floats2half2_rn(w.z * ic, w.w * ic);
+            p = make_uint2(*reinterpret_cast<const unsigned*>(&a), *reinterpret_cast<const unsigned*>(&b));
+        } else {
+            const __nv_bfloat162 a = __floats2bfloat162_rn(w.x * ic, w.y * ic),
+                                 b = __floats2bfloat162_rn(w.z * ic, w.w * ic);
+            p = make_uint2(*reinterpret_cast<const unsigned*>(&a), *reinterpret_cast<const unsigned*>(&b));
+        }
+        *reinterpret_cast<uint2*>(dst + 4 * k) = p;
+    };
+#pragma unroll
+    for (int i = 0; i < kQuantVec; ++i)
+        if (t + i * NT < nvec) store(t + i * NT, v[i]);
+    for (int k = t + kQuantVec * NT; k < nvec; k += NT) store(k, load(k));
+    if (t == 0) scale[row0 + r] = c;
 }
 
 // scatter-table arguments of the context (sigma_E^2 = kappa E)
@@ -1126,8 +1164,14 @@ lmosem_status hull_reset(lmosem_ctx* c, const WTabArgs& W, int n) {
 
 }  // namespace
 
+// Planes of every angle in the sensitivity's pass, while they are small enough.
+// At 50 x 50 (1.0 GB, 37k events) the whole reconstruction took 4.1 ms with
+// the fused pass and 4.3 without; at 64 x 64 (3.7 GB) the fused pass took 2.09 ms
+// and the planes' allocation 2.7 ms of host time, against 1.09 ms for the
+// sensitivity alone and 1.1 ms for k_wtable, which the grid form does without.
 bool wtab_all_fits(const lmosem_ctx* c) {
-    return (int64_t)c->n_angles * wtab_angle_floats(c) * (int64_t)sizeof(float) <= c->table_budget;
+    const int64_t bytes = (int64_t)c->n_angles * wtab_angle_floats(c) * (int64_t)sizeof(float);
+    return bytes <= std::min<int64_t>(c->table_budget, int64_t(1280) << 20) && c->n_scat <= 32 * 128;
 }
 
 lmosem_status wtab_all_with_sens(lmosem_ctx* c, double* sens_angle, float w_const_sens, float de0) {
@@ -1149,17 +1193,18 @@ lmosem_status wtab_all_with_sens(lmosem_ctx* c, double* sens_angle, float w_cons
 }
 
 lmosem_status quantize_rows(lmosem_ctx* c, int64_t rows, int64_t row0) {
-    const int qthreads = 256;
-    const unsigned qblocks = (unsigned)((rows + qthreads / 32 - 1) / (qthreads / 32));
+    const bool narrow = c->ld_model <= 64 * 4 * kQuantVec;
+    auto launch = [&](auto kern, auto* out, float hmax) {
+        kern<<<(unsigned)rows, narrow ? 64 : 256, 0, c->stream>>>(c->d_stage, c->ld_model, c->n_sup, c->ld_model, out,
+                                                                  row0, c->d_scale, hmax);
+    };
     LMOSEM_PROF_BEGIN(c);
     if (c->fmt == LMOSEM_MODEL_FP16_SCALED)
-        k_quantize<__half><<<qblocks, qthreads, 0, c->stream>>>(c->d_stage, c->ld_model, rows, c->n_sup, c->ld_model,
-                                                                reinterpret_cast<__half*>(c->d_model), row0,
-                                                                c->d_scale, 32768.0f);
+        launch(narrow ? k_quantize<__half, 64> : k_quantize<__half, 256>, reinterpret_cast<__half*>(c->d_model),
+               32768.0f);
     else
-        k_quantize<__nv_bfloat16><<<qblocks, qthreads, 0, c->stream>>>(
-            c->d_stage, c->ld_model, rows, c->n_sup, c->ld_model, reinterpret_cast<__nv_bfloat16*>(c->d_model), row0,
-            c->d_scale, 1.0f);
+        launch(narrow ? k_quantize<__nv_bfloat16, 64> : k_quantize<__nv_bfloat16, 256>,
+               reinterpret_cast<__nv_bfloat16*>(c->d_model), 1.0f);
     LMOSEM_LAUNCHED(c, LMOSEM_K_QUANTIZE);
     return LMOSEM_OK;
 }
