@@ -303,6 +303,18 @@ __device__ __forceinline__ float sum8_in_order(const float* v) {
     return y;
 }
 
+// FP64 sum over the block (at most 1024 threads, whole warps), in a fixed
+// order; every thread gets it.  sh: 32 doubles.
+__device__ __forceinline__ double block_sum(double v, double* sh) {
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();  // sh may be in use from an earlier sum
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double s = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh[w];
+    return s;
+}
+
 // ---- host entry points implemented in the other translation units
 lmosem_status build_tables(lmosem_ctx* c);                      // siddon.cu
 // h_offsets: n_real + 1 event offsets of the realisations (nullptr: one)

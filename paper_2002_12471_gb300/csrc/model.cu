@@ -160,11 +160,16 @@ struct WSensArgs {
     double* sens_angle;   // [a][n]
 };
 
-__global__ void k_wtable_sens(WSensArgs S) {
+// Blocks of kFuseX columns x kFuseY shares: share y takes the 32-pixel pieces
+// y, y + kFuseY, ... of the scatter pixels (the FP32 sums of a piece go
+// through shared memory and are added in order), so that a small problem
+// fills more than a few warps (16 x 16: 110 us with one share).
+constexpr int kFuseX = 64, kFuseY = 8;
+__global__ void __launch_bounds__(kFuseX * kFuseY) k_wtable_sens(WSensArgs S) {
+    extern __shared__ float pieces[];  // [piece][kFuseX]
     const WTabArgs& A = S.w;
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+    const int n = blockIdx.x * kFuseX + threadIdx.x;  // ld_w is a multiple of kTN, so of kFuseX
     const int a = blockIdx.y;
-    if (n >= A.ld_w) return;  // never splits a warp: ld_w is a multiple of kTN
     const size_t plane = (size_t)A.n_scat * A.ld_w;
     float* base = A.wtab + (size_t)a * 3 * plane + n;
     uint2* hull = A.hull + ((size_t)a * A.n_ptiles + n / kTN) * A.n_scat;
@@ -172,45 +177,45 @@ __global__ void k_wtable_sens(WSensArgs S) {
     const int pn = real ? A.sup[n] : 0;
     const float xn = pixel_x(pn, A.nx, A.dpx), yn = pixel_y(pn, A.nx, A.ny, A.dpx);
     const float2 trig = A.trig[a];
-    double acc = 0.0;
-    if (real)
-        acc = (double)(expf(-A.l_edge[(size_t)a * A.npix + pn]) * S.ppar[(size_t)a * A.ld_w + n].w * S.de0);
     const float* lp = A.l_pair + (real ? n : 0);
     const float* le = A.l_edge + (size_t)a * A.npix;
     const float* du = S.du_m + (size_t)a * A.n_scat;
-    float part = 0.0f;
-    for (int k = 0; k < A.n_scat; ++k) {
-        const float4 gm = __ldg(A.scat_geo + k);
-        const int pm = __float_as_int(gm.w);
-        float s = 0.0f, b = 0.0f, nlw = INFINITY;
-        uint2 hb = make_uint2(0xffffffffu, 0xffffffffu);
-        float cpsi, rinv;
-        if (real && path_geometry_xy(xn, yn, gm.x, gm.y, pn == pm, trig, &cpsi, &rinv)) {
-            float P, kt;
-            compton(cpsi, A.eps0, A.inv_kbar, &P, &kt);
-            const float2 cr = compton_lookup(A.compton, cpsi);  // (mu ratio, window mass)
-            const float att = fmaf(cr.x, __ldg(le + pm), lp[(size_t)k * A.n_sup]);
-            const float mu = gm.z;
-            const float e1 = A.e0 * P;
-            const float ri = rsqrtf(e1);
-            nlw = fmaf(att, kLog2e, -__log2f(A.w_const * mu * kt * rinv * ri));
-            s = A.cE * ri;
-            b = -e1 * s;
-            hb = hull_bits(e1, ri, A.hK);
-            const float w = S.w_const_sens * mu * kt * rinv * __expf(-att);
-            part = fmaf(w, __ldg(du + k) * cr.y, part);
+    const int n_pieces = (A.n_scat + 31) / 32;
+    for (int p = threadIdx.y; p < n_pieces; p += kFuseY) {
+        float part = 0.0f;
+        for (int k = 32 * p; k < min(A.n_scat, 32 * p + 32); ++k) {
+            const float4 gm = __ldg(A.scat_geo + k);
+            const int pm = __float_as_int(gm.w);
+            float s = 0.0f, b = 0.0f, nlw = INFINITY;
+            uint2 hb = make_uint2(0xffffffffu, 0xffffffffu);
+            float cpsi, rinv;
+            if (real && path_geometry_xy(xn, yn, gm.x, gm.y, pn == pm, trig, &cpsi, &rinv)) {
+                float P, kt;
+                compton(cpsi, A.eps0, A.inv_kbar, &P, &kt);
+                const float2 cr = compton_lookup(A.compton, cpsi);  // (mu ratio, window mass)
+                const float att = fmaf(cr.x, __ldg(le + pm), lp[(size_t)k * A.n_sup]);
+                const float mu = gm.z;
+                const float e1 = A.e0 * P;
+                const float ri = rsqrtf(e1);
+                nlw = fmaf(att, kLog2e, -__log2f(A.w_const * mu * kt * rinv * ri));
+                s = A.cE * ri;
+                b = -e1 * s;
+                hb = hull_bits(e1, ri, A.hK);
+                const float w = S.w_const_sens * mu * kt * rinv * __expf(-att);
+                part = fmaf(w, __ldg(du + k) * cr.y, part);
+            }
+            base[(size_t)k * A.ld_w] = s;
+            base[plane + (size_t)k * A.ld_w] = b;
+            base[2 * plane + (size_t)k * A.ld_w] = nlw;
+            hull_fold(hull + k, hb);
         }
-        base[(size_t)k * A.ld_w] = s;
-        base[plane + (size_t)k * A.ld_w] = b;
-        base[2 * plane + (size_t)k * A.ld_w] = nlw;
-        hull_fold(hull + k, hb);
-        if ((k & 31) == 31) {
-            acc += (double)part;
-            part = 0.0f;
-        }
+        pieces[p * kFuseX + threadIdx.x] = part;
     }
-    acc += (double)part;
-    if (real) S.sens_angle[(size_t)a * A.n_sup + n] = acc;
+    __syncthreads();
+    if (threadIdx.y != 0 || !real) return;
+    double acc = (double)(expf(-A.l_edge[(size_t)a * A.npix + pn]) * S.ppar[(size_t)a * A.ld_w + n].w * S.de0);
+    for (int p = 0; p < n_pieces; ++p) acc += (double)pieces[p * kFuseX + threadIdx.x];
+    S.sens_angle[(size_t)a * A.n_sup + n] = acc;
 }
 
 struct PathSumArgs {
@@ -1186,8 +1191,8 @@ lmosem_status wtab_all_with_sens(lmosem_ctx* c, double* sens_angle, float w_cons
     S.de0 = de0;
     S.sens_angle = sens_angle;
     LMOSEM_PROF_BEGIN(c);
-    // 64-thread blocks: every (column block, angle) resident at once
-    k_wtable_sens<<<dim3((c->ld_w + 63) / 64, c->n_angles), 64, 0, c->stream>>>(S);
+    const size_t smem = sizeof(float) * kFuseX * ((c->n_scat + 31) / 32);
+    k_wtable_sens<<<dim3(c->ld_w / kFuseX, c->n_angles), dim3(kFuseX, kFuseY), smem, c->stream>>>(S);
     LMOSEM_LAUNCHED(c, LMOSEM_K_SENS);
     return LMOSEM_OK;
 }

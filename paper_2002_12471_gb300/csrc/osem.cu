@@ -584,38 +584,26 @@ __global__ void k_subset_totals(const double* __restrict__ sens, int n_sup, cons
     }
 }
 
-// loglik = sum of the per-CTA partials - T sum_q s_q f_q (FP64, one block)
-__global__ void k_ll_final(const double* __restrict__ llpart, int nparts,
-                           const double* __restrict__ s_total, const float* __restrict__ f,
-                           int n_sup, double T, double* __restrict__ out) {
-    __shared__ double sh[256];
-    double acc = 0.0;
-    for (int n = threadIdx.x; n < n_sup; n += blockDim.x) acc += s_total[n] * (double)f[n];
-    sh[threadIdx.x] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double sf = 0.0;
-        for (int k = 0; k < (int)blockDim.x; ++k) sf += sh[k];
-        double ll = 0.0;
-        for (int k = 0; k < nparts; ++k) ll += llpart[k];
-        *out = ll - T * sf;
-    }
+// loglik = sum of the per-CTA partials - T sum_q s_q f_q (FP64, one block;
+// 60 us when one thread added the partials one load after the other)
+__global__ void __launch_bounds__(1024) k_ll_final(const double* __restrict__ llpart, int nparts,
+                                                   const double* __restrict__ s_total, const float* __restrict__ f,
+                                                   int n_sup, double T, double* __restrict__ out) {
+    __shared__ double sh[32];
+    double sf = 0.0, ll = 0.0;
+    for (int n = threadIdx.x; n < n_sup; n += blockDim.x) sf += s_total[n] * (double)f[n];
+    for (int k = threadIdx.x; k < nparts; k += blockDim.x) ll += llpart[k];
+    sf = block_sum(sf, sh);
+    ll = block_sum(ll, sh);
+    if (threadIdx.x == 0) *out = ll - T * sf;
 }
 
-__global__ void k_init_image(const double* __restrict__ s_total, int n_sup, double J, double T,
-                             float* __restrict__ f) {
-    __shared__ double sh[256];
+__global__ void __launch_bounds__(1024) k_init_image(const double* __restrict__ s_total, int n_sup, double J, double T,
+                                                     float* __restrict__ f) {
+    __shared__ double sh[32];
     double acc = 0.0;
     for (int n = threadIdx.x; n < n_sup; n += blockDim.x) acc += s_total[n];
-    sh[threadIdx.x] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int k = 0; k < (int)blockDim.x; ++k) s += sh[k];
-        sh[0] = s;
-    }
-    __syncthreads();
-    float v = (float)(J / (T * sh[0]));
+    const float v = (float)(J / (T * block_sum(acc, sh)));
     for (int n = threadIdx.x; n < n_sup; n += blockDim.x) f[n] = v;
 }
 
@@ -1378,7 +1366,7 @@ lmosem_status run_coop(lmosem_ctx* c, int n_iters, double T, float* d_f) {
 
 lmosem_status ll_final(lmosem_ctx* c, double T, const float* d_f, double* out) {
     LMOSEM_PROF_BEGIN(c);
-    k_ll_final<<<1, 256, 0, c->stream>>>(c->d_llpart, c->pass_grid,
+    k_ll_final<<<1, 1024, 0, c->stream>>>(c->d_llpart, c->pass_grid,
                                          c->d_sens + (size_t)c->n_subsets * c->n_sup, d_f,
                                          c->n_sup, T, out);
     LMOSEM_LAUNCHED(c, LMOSEM_K_UPDATE);
@@ -1506,7 +1494,7 @@ lmosem_status run_subset_totals(lmosem_ctx* c, double T, const float* d_f, doubl
 
 lmosem_status run_init_image(lmosem_ctx* c, double T, float* d_f) {
     LMOSEM_PROF_BEGIN(c);
-    k_init_image<<<1, 256, 0, c->stream>>>(c->d_sens + (size_t)c->sens_subsets * c->n_sup,
+    k_init_image<<<1, 1024, 0, c->stream>>>(c->d_sens + (size_t)c->sens_subsets * c->n_sup,
                                            c->n_sup, c->d_weight ? c->n_counts : (double)c->J, T, d_f);
     LMOSEM_LAUNCHED(c, LMOSEM_K_OTHER);
     return LMOSEM_OK;

@@ -71,17 +71,24 @@ __global__ void k_sens_angle(SensArgs A) {
     A.sens_angle[(size_t)a * A.n_sup + n] = acc;
 }
 
-__global__ void k_sens_reduce(const double* __restrict__ sens_angle, int n_angles, int n_sup,
-                              int n_subsets, double* __restrict__ sens, double* __restrict__ total) {
-    int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= n_sup) return;
+// s^i: a thread per (support pixel, subset) adds the subset's angles in order;
+// then one thread per pixel adds the subsets in order.
+constexpr int kRedSub = 8;
+__global__ void __launch_bounds__(32 * kRedSub) k_sens_reduce(const double* __restrict__ sens_angle, int n_angles,
+                                                              int n_sup, int n_subsets, double* __restrict__ sens,
+                                                              double* __restrict__ total) {
+    const int n = blockIdx.x * 32 + (threadIdx.x & 31);
+    if (n < n_sup)
+        for (int i = threadIdx.x >> 5; i < n_subsets; i += kRedSub) {
+            double s = 0.0;
+#pragma unroll 8
+            for (int a = i; a < n_angles; a += n_subsets) s += sens_angle[(size_t)a * n_sup + n];
+            sens[(size_t)i * n_sup + n] = s;
+        }
+    __syncthreads();
+    if (threadIdx.x >= 32 || n >= n_sup) return;
     double tot = 0.0;
-    for (int i = 0; i < n_subsets; ++i) {
-        double s = 0.0;
-        for (int a = i; a < n_angles; a += n_subsets) s += sens_angle[(size_t)a * n_sup + n];
-        sens[(size_t)i * n_sup + n] = s;
-        tot += s;
-    }
+    for (int i = 0; i < n_subsets; ++i) tot += sens[(size_t)i * n_sup + n];
     total[n] = tot;
 }
 
@@ -126,7 +133,7 @@ lmosem_status compute_sensitivity(lmosem_ctx* c, int n_subsets) {
     }
     // rows 0..n_subsets-1: s^i; row n_subsets: s = sum_i s^i
     LMOSEM_PROF_BEGIN(c);
-    k_sens_reduce<<<(c->n_sup + 255) / 256, 256, 0, c->stream>>>(
+    k_sens_reduce<<<(c->n_sup + 31) / 32, 32 * kRedSub, 0, c->stream>>>(
         c->d_sens_angle, c->n_angles, c->n_sup, n_subsets, c->d_sens,
         c->d_sens + (size_t)n_subsets * c->n_sup);
     LMOSEM_LAUNCHED(c, LMOSEM_K_SENS);

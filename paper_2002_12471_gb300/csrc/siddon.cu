@@ -194,7 +194,8 @@ lmosem_status build_tables(lmosem_ctx* c) {
                                  cudaMemcpyHostToDevice, c->stream));
     // the cos(psi) table on the device (FP64; 16k nodes would cost the host ~1 ms)
     LMOSEM_PROF_BEGIN(c);
-    k_compton_table<<<(kComptonNodes + 255) / 256, 256, 0, c->stream>>>(c->e0, c->fwhm_frac, c->e_lo, c->e_hi,
+    // one warp per CTA: 513 CTAs, so that the FP64 units of every SM take part
+    k_compton_table<<<(kComptonNodes + 31) / 32, 32, 0, c->stream>>>(c->e0, c->fwhm_frac, c->e_lo, c->e_hi,
                                                                          sig0, c->d_compton);
     LMOSEM_LAUNCHED(c, LMOSEM_K_TABLES);
 
