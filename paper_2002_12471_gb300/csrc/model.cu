@@ -911,12 +911,16 @@ __global__ void __launch_bounds__(NT) k_quantize(const float* __restrict__ stage
 //             + sum_m M_u(b; u_m) W_a(n, m) M_E(k; E'_a(n, m)).
 // For one (a, k) the scatter part is a product over m of the position-bin
 // masses (bins x scatter pixels) with C_k = W M_E (scatter pixels x support
-// pixels).  A CTA owns 64 position bins x 128 support pixels of one (a, k).
-// For each stage of 16 scatter pixels it forms C_k from the (s, b, -lw)
-// planes (sigma_E sqrt(2 pi) = sqrt(pi log2 e) / s, E' = -b / s, and
-// (E - E') / (sigma_E sqrt 2) = (E s + b) sqrt(ln 2)) and the bin masses from
-// the position parameters, then accumulates 8 bins x 4 pixels per thread; a
-// warp skips the scatter pixels whose cut misses all 8 of its bins.
+// pixels).  The complementary error functions of the masses bound the kernel
+// (about 45 instructions each, against one multiply-add per term), so each is
+// formed once: the position masses in a table per angle (k_bin_masses), and a
+// CTA forms C_k of up to 3 energy bins together from the masses' common edges.
+// A CTA owns 64 position bins x 128 support pixels of one angle and those
+// energy bins.  For each stage of 16 scatter pixels it forms C_k from the
+// (s, b, -lw) planes (sigma_E sqrt(2 pi) = sqrt(pi log2 e) / s, E' = -b / s, and
+// (E - E') / (sigma_E sqrt 2) = (E s + b) sqrt(ln 2)), then accumulates 4 bins x
+// 4 pixels x energy bins per thread; a warp skips the scatter pixels whose cut
+// misses all 4 of its bins.
 constexpr int kMaxEBins = 8;
 constexpr float kSqrtLn2 = 0.83255461115769776f;     // q sqrt(ln 2) = 1 / (sigma sqrt 2)
 constexpr float kSqrtPiLog2e = 2.1289340388624524f;  // sigma sqrt(2 pi) = sqrt(pi log2 e) / q
@@ -933,7 +937,8 @@ struct BinnedArgs {
     int n_ebins;
     float e_edge[kMaxEBins + 1];  // energy bin edges
     float pe_mass[kMaxEBins];     // photopeak mass of each energy bin
-    int n_btiles, n_ptiles;
+    const float* mass;            // position masses [a - a0][m][n_btiles x 64]
+    int n_btiles, n_ptiles, n_kgroups;
     const int32_t* rowmap;        // [a][b][k] -> sorted row, or -1
     float* out;
     int64_t ld_out;
@@ -941,31 +946,49 @@ struct BinnedArgs {
     int scatter_only;
 };
 
-// mass of a unit Gaussian on [zl, zh] in units of sigma sqrt 2, keeping its
-// relative accuracy far out in either tail
+// mass of a unit Gaussian on [zl, zh] in units of sigma sqrt 2 from el =
+// erfc(|zl|) and eh = erfc(|zh|), keeping its relative accuracy far out in
+// either tail
+__device__ __forceinline__ float edge_mass(float zl, float el, float zh, float eh) {
+    if (zl >= 0.0f) return 0.5f * (el - eh);
+    if (zh <= 0.0f) return 0.5f * (eh - el);
+    return 1.0f - 0.5f * (el + eh);
+}
 __device__ __forceinline__ float bin_mass(float zl, float zh) {
-    if (zl >= 0.0f) return 0.5f * (erfcf(zl) - erfcf(zh));
-    if (zh <= 0.0f) return 0.5f * (erfcf(-zh) - erfcf(-zl));
-    return 1.0f - 0.5f * (erfcf(-zl) + erfcf(zh));
+    return edge_mass(zl, erfcf(fabsf(zl)), zh, erfcf(fabsf(zh)));
 }
 
-constexpr int kBOffPlanes = 0;                          // [2][3][kStage][kTN]
-constexpr int kBOffMp = kBOffPlanes + 2 * 3 * kPlaneF;  // [2][kStage] float4
-constexpr int kBOffC = kBOffMp + 2 * kStage * 4;        // [kStage][kTN]  C_k of the stage
-constexpr int kBOffM = kBOffC + kStage * kTN;           // [kStage][kTJ]  bin masses of the stage
-constexpr int kBOffMisc = kBOffM + kStage * kTJ;        // 16 ints
-constexpr int kBOffList = kBOffMisc + 16;               // n_scat ints
+// position masses of every (scatter pixel, detector bin) of angles a0 ..;
+// zero beyond the position cut and for padding bins
+__global__ void k_bin_masses(const float4* __restrict__ mpar, int n_scat, int a0, int n_bins, int nb_pad, float bin_mm,
+                             float half, float* __restrict__ mass) {
+    const int m = blockIdx.x, a = a0 + blockIdx.y;
+    const float4 q = mpar[(size_t)a * n_scat + m];
+    const float s2 = q.y * kSqrtLn2;
+    for (int b = threadIdx.x; b < nb_pad; b += blockDim.x) {
+        const float ulo = -half + b * bin_mm, uhi = ulo + bin_mm;
+        const float dn = q.x < ulo ? ulo - q.x : (q.x > uhi ? q.x - uhi : 0.0f);
+        mass[((size_t)blockIdx.y * n_scat + m) * nb_pad + b] =
+            (b < n_bins && dn <= q.w) ? bin_mass((ulo - q.x) * s2, (uhi - q.x) * s2) : 0.0f;
+    }
+}
 
-__global__ void __launch_bounds__(kBuildThreads, 2) k_binned(BinnedArgs A) {
+constexpr int kBinThreads = 512, kBinWarps = kBinThreads / 32, kBinRows = kTJ / kBinWarps;  // 4 bins per warp
+constexpr int kBOffPlanes = 0;                             // [2][3][kStage][kTN]
+constexpr int kBOffM = kBOffPlanes + 2 * 3 * kPlaneF;      // [2][kStage][kTJ]  bin masses of the stage
+constexpr int kBOffC = kBOffM + 2 * kStage * kTJ;          // [kGroup][kStage][kTN]  C_k of the stage
+constexpr int kBinGroup = 3;                               // energy bins per CTA at most
+static_assert(kBinRows == 4, "one float4 of masses per warp and scatter pixel");
+
+template <int KG>
+__global__ void __launch_bounds__(kBinThreads, 1) k_binned(BinnedArgs A) {
     extern __shared__ float4 smem4[];
     float* sm = reinterpret_cast<float*>(smem4);
     float* planes = sm + kBOffPlanes;
-    float4* mp = reinterpret_cast<float4*>(sm + kBOffMp);
-    float* Cm = sm + kBOffC;
     float* Mb = sm + kBOffM;
-    int* misc = reinterpret_cast<int*>(sm + kBOffMisc);
-    unsigned* live = reinterpret_cast<unsigned*>(misc) + 8;
-    int* mlist = reinterpret_cast<int*>(sm + kBOffList);
+    float* Cm = sm + kBOffC;
+    int* misc = reinterpret_cast<int*>(Cm + KG * kStage * kTN);
+    int* mlist = misc + kBinWarps;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     int idx = blockIdx.x;
@@ -973,22 +996,22 @@ __global__ void __launch_bounds__(kBuildThreads, 2) k_binned(BinnedArgs A) {
     idx /= A.n_ptiles;
     const int bt = idx % A.n_btiles;
     idx /= A.n_btiles;
-    const int k = idx % A.n_ebins;
-    const int a = A.a0 + idx / A.n_ebins;
-    const int b0 = bt * kTJ, n0 = pt * kTN;
+    const int k0 = idx % A.n_kgroups * KG;
+    const int ai = idx / A.n_kgroups, a = A.a0 + ai;
+    const int b0 = bt * kTJ, n0 = pt * kTN, nk = min(KG, A.n_ebins - k0);
     const int nb = min(kTJ, A.n_bins - b0);
-    const int32_t* rmap = A.rowmap + (size_t)a * A.n_bins * A.n_ebins + k;
+    const int32_t* rmap = A.rowmap + (size_t)a * A.n_bins * A.n_ebins + k0;
 
     // nothing to do unless one of the CTA's bins holds a row
     bool has = false;
-    for (int bl = tid; bl < nb; bl += kBuildThreads) has |= rmap[(size_t)(b0 + bl) * A.n_ebins] >= 0;
+    for (int bl = tid; bl < nb * nk; bl += kBinThreads) has |= rmap[(size_t)(b0 + bl / nk) * A.n_ebins + bl % nk] >= 0;
     if (!__syncthreads_or(has)) return;
 
     // scatter pixels whose cut interval reaches the CTA's bins
     const float umin = -A.half + b0 * A.bin_mm, umax = -A.half + (b0 + nb) * A.bin_mm;
     const float4* mp_a = A.mpar + (size_t)a * A.n_scat;
     int nm = 0;
-    for (int m0 = 0; m0 < A.n_scat; m0 += kBuildThreads) {
+    for (int m0 = 0; m0 < A.n_scat; m0 += kBinThreads) {
         const int m = m0 + tid;
         bool in = false;
         if (m < A.n_scat) {
@@ -999,7 +1022,7 @@ __global__ void __launch_bounds__(kBuildThreads, 2) k_binned(BinnedArgs A) {
         if (lane == 0) misc[warp] = __popc(bal);
         __syncthreads();
         int off = nm, total = 0;
-        for (int w = 0; w < kBuildThreads / 32; ++w) {
+        for (int w = 0; w < kBinWarps; ++w) {
             const int cw = misc[w];
             if (w < warp) off += cw;
             total += cw;
@@ -1009,108 +1032,127 @@ __global__ void __launch_bounds__(kBuildThreads, 2) k_binned(BinnedArgs A) {
         nm += total;
     }
 
-    // primary path: w_0 M_u(b; u_n) M_E(k; E0), 8 bins x 4 pixels per thread
-    float2 acc[8][2];
+    // primary path: w_0 M_u(b; u_n) M_E(k; E0), 4 bins x 4 pixels per thread
+    float2 acc[KG][kBinRows][2];
     {
         const float4* pp_a = A.ppar + (size_t)a * A.ld_w + n0 + 4 * lane;
         float w0[4], s2[4], un[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const float4 pp = __ldg(pp_a + q);
-            w0[q] = (pp.y > 0.0f && !A.scatter_only) ? ex2_approx(pp.z) * kSqrtPiLog2e / pp.y * A.pe_mass[k]
-                                                     : 0.0f;
+            w0[q] = (pp.y > 0.0f && !A.scatter_only) ? ex2_approx(pp.z) * kSqrtPiLog2e / pp.y : 0.0f;
             s2[q] = pp.y * kSqrtLn2;
             un[q] = pp.x;
         }
 #pragma unroll
-        for (int jj = 0; jj < 8; ++jj) {
-            const int b = b0 + 8 * warp + jj;
+        for (int jj = 0; jj < kBinRows; ++jj) {
+            const int b = b0 + kBinRows * warp + jj;
             const float ulo = -A.half + b * A.bin_mm, uhi = ulo + A.bin_mm;
             float v[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-                v[q] = (b < A.n_bins && w0[q] != 0.0f)
-                           ? w0[q] * bin_mass((ulo - un[q]) * s2[q], (uhi - un[q]) * s2[q])
-                           : 0.0f;
-            acc[jj][0] = make_float2(v[0], v[1]);
-            acc[jj][1] = make_float2(v[2], v[3]);
+                v[q] = (b < A.n_bins && w0[q] != 0.0f) ? bin_mass((ulo - un[q]) * s2[q], (uhi - un[q]) * s2[q]) : 0.0f;
+#pragma unroll
+            for (int g = 0; g < KG; ++g) {
+                const float pe = k0 + g < A.n_ebins ? A.pe_mass[k0 + g] : 0.0f;
+                acc[g][jj][0] = make_float2(w0[0] * pe * v[0], w0[1] * pe * v[1]);
+                acc[g][jj][1] = make_float2(w0[2] * pe * v[2], w0[3] * pe * v[3]);
+            }
         }
     }
 
     const size_t plane = (size_t)A.n_scat * A.ld_w;
-    const int slot = A.wslot_by_angle ? a : a - A.a0;
-    const float* tab = A.wtab + (size_t)slot * 3 * plane + n0;
-    TileInfo T;
-    T.nm = nm;
-    const float el = A.e_edge[k], eh = A.e_edge[k + 1];
+    const float* tab = A.wtab + (size_t)(A.wslot_by_angle ? a : ai) * 3 * plane + n0;
+    const float* mass = A.mass + (size_t)ai * A.n_scat * (A.n_btiles * kTJ) + b0;
+    float edge[KG + 1];
+#pragma unroll
+    for (int g = 0; g <= KG; ++g) edge[g] = A.e_edge[min(k0 + g, A.n_ebins)];
     const int nchunks = (nm + kStage - 1) / kStage;
-    if (nchunks > 0) stage_issue(T, mlist, tab, plane, A.ld_w, mp_a, planes, mp, 0, 0, kTN / 4);
+    // stage c of the strip union into buffer buf: planes and masses (padded
+    // scatter pixels: w = inf and no mass, i.e. exact zeros)
+    auto issue = [&](int c, int buf) {
+        for (int k = tid; k < 3 * kStage * (kTN / 4); k += kBinThreads) {
+            const int p = k / (kStage * (kTN / 4)), r = k % (kStage * (kTN / 4)), mc = r / (kTN / 4), q = r % (kTN / 4);
+            float* dst = planes + ((buf * 3 + p) * kStage + mc) * kTN + 4 * q;
+            if (c * kStage + mc < nm) {
+                cp_async16(dst, tab + p * plane + (size_t)mlist[c * kStage + mc] * A.ld_w + 4 * q);
+            } else {
+                const float v = p == 2 ? INFINITY : 0.0f;
+                *reinterpret_cast<float4*>(dst) = make_float4(v, v, v, v);
+            }
+        }
+        if (tid < kStage * (kTJ / 4)) {
+            const int mc = tid / (kTJ / 4), q = tid % (kTJ / 4);
+            float* dst = Mb + (buf * kStage + mc) * kTJ + 4 * q;
+            if (c * kStage + mc < nm) cp_async16(dst, mass + (size_t)mlist[c * kStage + mc] * (A.n_btiles * kTJ) + 4 * q);
+            else *reinterpret_cast<float4*>(dst) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+        cp_async_commit();
+    };
+    if (nchunks > 0) issue(0, 0);
     for (int c = 0; c < nchunks; ++c) {
         const int buf = c & 1;
-        if (tid < kBuildThreads / 32) live[tid] = 0u;
         if (c + 1 < nchunks) {
-            stage_issue(T, mlist, tab, plane, A.ld_w, mp_a, planes, mp, (c + 1) * kStage, buf ^ 1, kTN / 4);
+            issue(c + 1, buf ^ 1);
             cp_async_wait<1>();
         } else {
             cp_async_wait<0>();
         }
         __syncthreads();
-        // bin masses of the stage: lanes hold bins 32 (warp & 1) + lane of one mc
-        for (int kk = tid; kk < kStage * kTJ; kk += kBuildThreads) {
-            const int mc = kk / kTJ, bl = kk - mc * kTJ;
-            const float4 q = mp[buf * kStage + mc];
-            const float ulo = -A.half + (b0 + bl) * A.bin_mm, uhi = ulo + A.bin_mm;
-            const float dn = q.x < ulo ? ulo - q.x : (q.x > uhi ? q.x - uhi : 0.0f);
-            const float s2 = q.y * kSqrtLn2;
-            const float M = (bl < nb && dn <= q.w) ? bin_mass((ulo - q.x) * s2, (uhi - q.x) * s2) : 0.0f;
-            Mb[mc * kTJ + bl] = M;
-            const unsigned bal = __ballot_sync(0xffffffffu, M != 0.0f);
-            if (lane < 4 && ((bal >> (8 * lane)) & 0xffu)) atomicOr(live + 4 * (warp & 1) + lane, 1u << mc);
-        }
         // C_k = W M_E(k; E') of the stage
         const float* pS = planes + (buf * 3 + 0) * kPlaneF;
         const float* pB = planes + (buf * 3 + 1) * kPlaneF;
         const float* pW = planes + (buf * 3 + 2) * kPlaneF;
-        for (int kk = tid; kk < kStage * kTN; kk += kBuildThreads) {
+#pragma unroll
+        for (int kk = tid; kk < kStage * kTN; kk += kBinThreads) {
             const float sv = pS[kk], bv = pB[kk], nlw = pW[kk];
-            float Cv = 0.0f;
-            if (sv > 0.0f && nlw < INFINITY)
-                Cv = ex2_approx(-nlw) * kSqrtPiLog2e / sv *
-                     bin_mass(fmaf(el, sv, bv) * kSqrtLn2, fmaf(eh, sv, bv) * kSqrtLn2);
-            Cm[kk] = Cv;
+            const bool on = sv > 0.0f && nlw < INFINITY;
+            const float w = on ? ex2_approx(-nlw) * kSqrtPiLog2e / sv : 0.0f;
+            float zl = fmaf(edge[0], sv, bv) * kSqrtLn2, el = erfcf(fabsf(zl));
+#pragma unroll
+            for (int g = 0; g < KG; ++g) {
+                const float zh = fmaf(edge[g + 1], sv, bv) * kSqrtLn2, eh = erfcf(fabsf(zh));
+                Cm[g * kStage * kTN + kk] = on ? w * edge_mass(zl, el, zh, eh) : 0.0f;
+                zl = zh;
+                el = eh;
+            }
         }
         __syncthreads();
-        const unsigned wlive = live[warp];
         for (int mc = 0; mc < kStage; ++mc) {
-            if (!((wlive >> mc) & 1u)) continue;
-            const float4 C = *reinterpret_cast<const float4*>(Cm + mc * kTN + 4 * lane);
-            const float4 M0 = *reinterpret_cast<const float4*>(Mb + mc * kTJ + 8 * warp);
-            const float4 M1 = *reinterpret_cast<const float4*>(Mb + mc * kTJ + 8 * warp + 4);
-            const float Mv[8] = {M0.x, M0.y, M0.z, M0.w, M1.x, M1.y, M1.z, M1.w};
-            const float2 C01 = make_float2(C.x, C.y), C23 = make_float2(C.z, C.w);
+            const float4 M = *reinterpret_cast<const float4*>(Mb + (buf * kStage + mc) * kTJ + kBinRows * warp);
+            if (M.x == 0.0f && M.y == 0.0f && M.z == 0.0f && M.w == 0.0f) continue;
+            const float Mv[kBinRows] = {M.x, M.y, M.z, M.w};
 #pragma unroll
-            for (int jj = 0; jj < 8; ++jj) {
-                const float2 m2 = make_float2(Mv[jj], Mv[jj]);
-                acc[jj][0] = ffma2(m2, C01, acc[jj][0]);
-                acc[jj][1] = ffma2(m2, C23, acc[jj][1]);
+            for (int g = 0; g < KG; ++g) {
+                const float4 C = *reinterpret_cast<const float4*>(Cm + (g * kStage + mc) * kTN + 4 * lane);
+                const float2 C01 = make_float2(C.x, C.y), C23 = make_float2(C.z, C.w);
+#pragma unroll
+                for (int jj = 0; jj < kBinRows; ++jj) {
+                    const float2 m2 = make_float2(Mv[jj], Mv[jj]);
+                    acc[g][jj][0] = ffma2(m2, C01, acc[g][jj][0]);
+                    acc[g][jj][1] = ffma2(m2, C23, acc[g][jj][1]);
+                }
             }
         }
         __syncthreads();
     }
 
+    const int n = n0 + 4 * lane;
 #pragma unroll
-    for (int jj = 0; jj < 8; ++jj) {
-        const int b = b0 + 8 * warp + jj;
-        if (b >= A.n_bins) continue;
-        const int32_t r = rmap[(size_t)b * A.n_ebins];
-        if (r >= 0) {
+    for (int g = 0; g < KG; ++g) {
+        if (k0 + g >= A.n_ebins) break;
+#pragma unroll
+        for (int jj = 0; jj < kBinRows; ++jj) {
+            const int b = b0 + kBinRows * warp + jj;
+            if (b >= A.n_bins) continue;
+            const int32_t r = rmap[(size_t)b * A.n_ebins + g];
+            if (r < 0) continue;
             float* row = A.out + (int64_t)r * A.ld_out;
-            const int n = n0 + 4 * lane;
             if (n + 3 < A.n_store) {
                 *reinterpret_cast<float4*>(row + n) =
-                    make_float4(acc[jj][0].x, acc[jj][0].y, acc[jj][1].x, acc[jj][1].y);
+                    make_float4(acc[g][jj][0].x, acc[g][jj][0].y, acc[g][jj][1].x, acc[g][jj][1].y);
             } else {
-                const float v[4] = {acc[jj][0].x, acc[jj][0].y, acc[jj][1].x, acc[jj][1].y};
+                const float v[4] = {acc[g][jj][0].x, acc[g][jj][0].y, acc[g][jj][1].x, acc[g][jj][1].y};
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                     if (n + q < A.n_store) row[n + q] = v[q];
@@ -1790,8 +1832,17 @@ lmosem_status build_binned_rows(lmosem_ctx* c, const int32_t* d_rowmap, int n_eb
                                      cudaMemcpyHostToDevice, c->stream));
         if ((st = dev_alloc(c, &c->d_wtab, (size_t)gsz * wtab_angle_floats(c)))) return st;
     }
-    const size_t smem = sizeof(float) * ((size_t)kBOffList + c->n_scat);
-    LMOSEM_CK(c, cudaFuncSetAttribute(k_binned, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int KG = std::min(kBinGroup, n_ebins), nb_pad = n_btiles * kTJ;
+    B.n_kgroups = (n_ebins + KG - 1) / KG;
+    auto kern = KG == 1 ? k_binned<1> : (KG == 2 ? k_binned<2> : k_binned<3>);
+    const size_t smem = sizeof(float) * ((size_t)kBOffC + KG * kStage * kTN + kBinWarps + c->n_scat);
+    LMOSEM_CK(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the mass tables of a launch: at most 256 MB
+    const int64_t mass_angle = (int64_t)c->n_scat * nb_pad;
+    const int msz = (int)std::max<int64_t>(1, std::min<int64_t>(gsz, (int64_t(1) << 26) / std::max<int64_t>(1, mass_angle)));
+    float* d_mass = nullptr;
+    Scratch tmp2(c);
+    if ((st = tmp2.alloc(&d_mass, (size_t)msz * mass_angle))) return st;
     for (int a0 = 0; a0 < c->n_angles; a0 += gsz) {
         const int na = std::min(gsz, c->n_angles - a0);
         if (!pre) {
@@ -1801,11 +1852,22 @@ lmosem_status build_binned_rows(lmosem_ctx* c, const int32_t* d_rowmap, int n_eb
             k_wtable<<<dim3((c->ld_w + 255) / 256, c->n_scat), 256, 0, c->stream>>>(W, na);
             LMOSEM_LAUNCHED(c, LMOSEM_K_WTABLE);
         }
-        B.wtab = pre ? c->d_wtab_all : c->d_wtab;
-        B.a0 = a0;
-        LMOSEM_PROF_BEGIN(c);
-        k_binned<<<(unsigned)((int64_t)na * n_ebins * n_btiles * n_ptiles), kBuildThreads, smem, c->stream>>>(B);
-        LMOSEM_LAUNCHED(c, LMOSEM_K_PATHSUM);
+        for (int a1 = a0; a1 < a0 + na; a1 += msz) {
+            const int nm = std::min(msz, a0 + na - a1);
+            if (c->n_scat > 0) {
+                LMOSEM_PROF_BEGIN(c);
+                k_bin_masses<<<dim3(c->n_scat, nm), 64, 0, c->stream>>>(c->d_mpar, c->n_scat, a1, c->n_bins, nb_pad,
+                                                                        B.bin_mm, B.half, d_mass);
+                LMOSEM_LAUNCHED(c, LMOSEM_K_WTABLE);
+            }
+            // planes indexed by angle, or by angle - a0 of the table group
+            B.wtab = pre ? c->d_wtab_all : c->d_wtab + (size_t)(a1 - a0) * 3 * c->n_scat * c->ld_w;
+            B.mass = d_mass;
+            B.a0 = a1;
+            LMOSEM_PROF_BEGIN(c);
+            kern<<<(unsigned)((int64_t)nm * B.n_kgroups * n_btiles * n_ptiles), kBinThreads, smem, c->stream>>>(B);
+            LMOSEM_LAUNCHED(c, LMOSEM_K_PATHSUM);
+        }
     }
     dev_free(c, &c->d_wtab);      // stream-ordered frees: no host wait
     dev_free(c, &c->d_wtab_all);  // consumed
