@@ -842,22 +842,32 @@ struct RowArgs {
 
 // Rows of 64 events (in block order) x 128 support pixels: the 13 x 9 grid
 // values around a block of 2 x 2 cells are loaded once for all of its events.
-// The loads bound the kernel (one L1 wavefront per value and warp): blocks of
-// 2 x 2 cells hold about twice the events of a cell for 1.2 times the values
-// (per 33k events x 5,884 pixels 1.97 -> 1.78 ms).  Slower: moving the values
-// of a neighbouring block up in registers (2.20 ms, 186 registers) and
-// prefetching the next block's lines to L1 (2.25 ms).
+// Instructions bound the kernel (about 250 issue slots per event and warp when
+// the stencil of an odd cell was copied to even registers): blocks of 2 x 2
+// cells hold about twice the events of a cell for 1.2 times the values (per 33k
+// events x 5,884 pixels 1.97 -> 1.78 ms), and an odd cell shifts its 12 weights
+// instead of 96 values (model build of 250k events at 128 x 128 50.0 -> 48.7 ms,
+// of 450k at 64 x 64 9.20 -> 8.57).  Slower: larger blocks (53.6 to 54.9 ms; 174
+// to 192 registers), two lanes per pixel (53.3; 20 warps per SM instead of 12),
+// the values of 8 blocks in shared memory (2.40 ms per 33k), those of a
+// neighbouring block moved up in registers (2.20), the next block's lines
+// prefetched to L1 (2.25).
 constexpr int kRowEvents = 64;
 template <int OX, int OU>
 __device__ __forceinline__ float stencil_sum(const float (&tv)[kPE + 1][kPU + 1], const float (&we)[kPE],
                                              const float (&wu)[kPU]) {
+    // pairs of values as they lie in the registers; OU = 1 shifts the weights
+    float2 w[kPU / 2];
+#pragma unroll
+    for (int k = 0; k < kPU; k += 2)
+        w[k / 2] = OU ? make_float2(k ? wu[k - 1] : 0.0f, wu[k]) : make_float2(wu[k], wu[k + 1]);
     float acc = 0.0f;
 #pragma unroll
     for (int q = 0; q < kPE; ++q) {
-        float2 v = make_float2(0.0f, 0.0f);
+        const float* t = tv[q + OX];
+        float2 v = make_float2(OU ? wu[kPU - 1] * t[kPU] : 0.0f, 0.0f);
 #pragma unroll
-        for (int k = 0; k < kPU; k += 2)
-            v = fma2(make_float2(wu[k], wu[k + 1]), make_float2(tv[q + OX][k + OU], tv[q + OX][k + OU + 1]), v);
+        for (int k = 0; k < kPU; k += 2) v = fma2(w[k / 2], make_float2(t[k], t[k + 1]), v);
         acc = fmaf(we[q], v.x + v.y, acc);
     }
     return acc;
