@@ -847,7 +847,8 @@ struct RowArgs {
 // cells hold about twice the events of a cell for 1.2 times the values (per 33k
 // events x 5,884 pixels 1.97 -> 1.78 ms), and an odd cell shifts its 12 weights
 // instead of 96 values (model build of 250k events at 128 x 128 50.0 -> 48.7 ms,
-// of 450k at 64 x 64 9.20 -> 8.57).  Slower: larger blocks (53.6 to 54.9 ms; 174
+// of 450k at 64 x 64 9.20 -> 8.57), and the sum over the energy nodes comes
+// first, packed throughout (48.7 -> 48.4, 8.57 -> 8.40).  Slower: larger blocks (53.6 to 54.9 ms; 174
 // to 192 registers), two lanes per pixel (53.3; 20 warps per SM instead of 12),
 // the values of 8 blocks in shared memory (2.40 ms per 33k), those of a
 // neighbouring block moved up in registers (2.20), the next block's lines
@@ -861,16 +862,23 @@ __device__ __forceinline__ float stencil_sum(const float (&tv)[kPE + 1][kPU + 1]
 #pragma unroll
     for (int k = 0; k < kPU; k += 2)
         w[k / 2] = OU ? make_float2(k ? wu[k - 1] : 0.0f, wu[k]) : make_float2(wu[k], wu[k + 1]);
-    float acc = 0.0f;
+    // over the energy nodes first: a position's chain is packed throughout
+    float2 v[kPU / 2];
+    float last = 0.0f;
+#pragma unroll
+    for (int k = 0; k < kPU / 2; ++k) v[k] = make_float2(0.0f, 0.0f);
 #pragma unroll
     for (int q = 0; q < kPE; ++q) {
         const float* t = tv[q + OX];
-        float2 v = make_float2(OU ? wu[kPU - 1] * t[kPU] : 0.0f, 0.0f);
+        const float2 e = make_float2(we[q], we[q]);
 #pragma unroll
-        for (int k = 0; k < kPU; k += 2) v = fma2(w[k / 2], make_float2(t[k], t[k + 1]), v);
-        acc = fmaf(we[q], v.x + v.y, acc);
+        for (int k = 0; k < kPU; k += 2) v[k / 2] = fma2(e, make_float2(t[k], t[k + 1]), v[k / 2]);
+        if (OU) last = fmaf(we[q], t[kPU], last);
     }
-    return acc;
+    float2 acc = make_float2(OU ? wu[kPU - 1] * last : 0.0f, 0.0f);
+#pragma unroll
+    for (int k = 0; k < kPU / 2; ++k) acc = fma2(w[k], v[k], acc);
+    return acc.x + acc.y;
 }
 __global__ void __launch_bounds__(128) k_grid_rows(RowArgs A) {
     __shared__ float4 sev[kRowEvents * 6];
