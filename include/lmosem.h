@@ -469,11 +469,12 @@ int64_t lmosem_model_bytes(const lmosem_ctx* ctx);
 /* Number of kernel launches this context has enqueued so far. */
 int64_t lmosem_launch_count(const lmosem_ctx* ctx);
 
-/* Path terms that the path-sum kernels formed in their last row build on
- * this context (paper Eq. 2 with Eq. 4: one term per (event, support pixel)
+/* Path terms of the last row build on this context (paper Eq. 2 with Eq. 4: one term per (event, support pixel)
  * for the primary path and one per (event, support pixel, scatter pixel)
  * whose term the position cut (k_sigma) and the energy cut (e_sigma) keep).
- * After lmosem_build_model or lmosem_build_model_batch with an FP32, FP16
+ * The path-sum kernels count them as they form them; for a build that formed
+ * the scatter sum on the grid (large event lists) they are counted when this
+ * is called, which takes about the time of the path sum.  After lmosem_build_model or lmosem_build_model_batch with an FP32, FP16
  * or BF16 format that is the whole model.  A surrogate build runs the path
  * sum on the rows its exact judge and energy gate recompute, one set of
  * rows at a time, and the count covers the last such set.  Padding columns
