@@ -494,8 +494,44 @@ __global__ void __launch_bounds__(kMaxPassThreads, pass_min_ctas<H, VPT>()) k_pa
     }
 }
 
-// b_q = sum of the per-CTA partials, then f_q <- f_q b_q / (T s^i_q), with
-// every SM busy: a CTA owns 8 support
+// b_q = sum of the per-CTA partials, then f_q <- f_q b_q / (T s^i_q).  One
+// CTA of kUpdWarps warps per 32 support pixels; warp w sums the partials
+// w, w + kUpdWarps, ... with eight loads in flight, then warp 0 adds the warp
+// sums in warp order (fixed order: deterministic).
+constexpr int kUpdWarps = 32;
+__global__ void __launch_bounds__(kUpdWarps * 32) k_update(const float* __restrict__ bpart, int nparts,
+                                                          int n_sup, float* __restrict__ f,
+                                                          const double* __restrict__ sens_i, double T,
+                                                          const int* __restrict__ status) {
+    if (status && *status) return;  // the pass was abandoned: keep the image
+    __shared__ float sh[kUpdWarps][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nw = blockDim.x >> 5;  // <= kUpdWarps
+    const int n = blockIdx.x * 32 + lane;
+    float b = 0.0f;
+    if (n < n_sup) {
+        int c = warp;
+        for (; c + 7 * nw < nparts; c += 8 * nw) {
+            float v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = bpart[(size_t)(c + k * nw) * n_sup + n];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) b += v[k];
+        }
+        for (; c < nparts; c += nw) b += bpart[(size_t)c * n_sup + n];
+    }
+    sh[warp][lane] = b;
+    __syncthreads();
+    if (warp == 0 && n < n_sup) {
+        float s = 0.0f;
+        for (int w = 0; w < nw; ++w) s += sh[w][lane];
+        double sd = sens_i[n];
+        float ts = (float)(T * sd);
+        f[n] = sd > 0.0 ? f[n] * s / ts : 0.0f;
+    }
+}
+
+// b_q over the per-CTA partials with every SM busy: a CTA owns 8 support
 // pixels, its 32 groups of 8 threads sum the partials g, g + 32, ... (one
 // 32-byte sector per load), then group 0 adds the 32 group sums in order.
 constexpr int kUpdPix = 8, kUpdGroups = 32;
@@ -1487,62 +1523,54 @@ constexpr int kNoAllocMaxDevices = 64;
 
 __device__ __align__(256) float g_noalloc_scratch[kNoAllocScratchFloats];
 
-// What the calls need of a device, looked up once: the array's address, its
-// SMs, and the CTAs per SM of every kernel and block size.  The driver queries
-// took about a third of a small call's host time.
-constexpr int kNoAllocWidths[] = {1, 2, 3, 4, 6, kNoAllocMaxVpt};
-constexpr int kNoAllocKernels = sizeof(kNoAllocWidths) / sizeof(int);
-struct NoAllocDevice {
-    float* scratch = nullptr;
-    int sms = 0;
-    int per_sm[kNoAllocKernels][kMaxPassThreads / 32 + 1] = {};
-};
 std::mutex g_noalloc_mu;
-NoAllocDevice g_noalloc[kNoAllocMaxDevices];
+float* g_noalloc_ptr[kNoAllocMaxDevices] = {};
 
 template <int VPT>
 inline auto noalloc_kernel() {
     return k_pass<float, VPT, VPT >= 6 ? 1 : (VPT >= 3 ? 2 : 4), true, false>;
 }
 
-// First call on a device: the look-ups above, which also load every kernel
-// this entry point can launch (module loading is lazy by default), so that
+// First call on a device: the array's address, and every kernel this entry
+// point can launch loaded now (module loading is lazy by default), so that
 // later calls with another row width load nothing.
-cudaError_t noalloc_setup(int dev) {
-    NoAllocDevice d;
+cudaError_t noalloc_setup() {
     void* p = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
+    cudaFuncAttributes fa;
     const void* kerns[] = {(const void*)noalloc_kernel<1>(), (const void*)noalloc_kernel<2>(),
                            (const void*)noalloc_kernel<3>(), (const void*)noalloc_kernel<4>(),
-                           (const void*)noalloc_kernel<6>(), (const void*)noalloc_kernel<kNoAllocMaxVpt>()};
-    for (int k = 0; k < kNoAllocKernels; ++k)
-        for (int w = 1; w <= kMaxPassThreads / 32; ++w)
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d.per_sm[k][w], kerns[k], 32 * w, 0)) != cudaSuccess)
-                return e;
-    cudaFuncAttributes fa;
-    if ((e = cudaFuncGetAttributes(&fa, k_update_px)) != cudaSuccess) return e;
-    d.scratch = static_cast<float*>(p);
-    g_noalloc[dev] = d;
+                           (const void*)noalloc_kernel<6>(), (const void*)noalloc_kernel<8>(),
+                           (const void*)k_update};
+    for (const void* k : kerns)
+        if ((e = cudaFuncGetAttributes(&fa, k)) != cudaSuccess) return e;
+    int dev = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    g_noalloc_ptr[dev] = static_cast<float*>(p);
     return cudaSuccess;
 }
 
-cudaError_t noalloc_device(const NoAllocDevice** out) {
+cudaError_t noalloc_scratch(float** out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kNoAllocMaxDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(g_noalloc_mu);
-    if (!g_noalloc[dev].scratch && (e = noalloc_setup(dev)) != cudaSuccess) return e;
-    *out = &g_noalloc[dev];
+    if (!g_noalloc_ptr[dev] && (e = noalloc_setup()) != cudaSuccess) return e;
+    *out = g_noalloc_ptr[dev];
     return cudaSuccess;
 }
 
 template <int VPT>
-cudaError_t noalloc_pass(const PassArgs& A0, int64_t rows, int nt, int sms, int per_sm, cudaStream_t s, int* grid_out) {
+cudaError_t noalloc_pass(const PassArgs& A0, int64_t rows, int nt, cudaStream_t s, int* grid_out) {
     constexpr int R = VPT >= 6 ? 1 : (VPT >= 3 ? 2 : 4);
     auto kern = noalloc_kernel<VPT>();
+    int per_sm = 0, dev = 0, sms = 0;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, 0);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
     PassArgs A = A0;
     int64_t grid = std::max(1, per_sm) * (int64_t)sms;
     grid = std::min<int64_t>(grid, kNoAllocScratchFloats / A.n_sup);
@@ -1553,7 +1581,7 @@ cudaError_t noalloc_pass(const PassArgs& A0, int64_t rows, int nt, int sms, int 
     kern<<<(unsigned)grid, nt, 0, s>>>(A);
     *grid_out = (int)grid;
     // no error was pending before the call, so one seen here is this launch's
-    cudaError_t e = cudaPeekAtLastError();
+    e = cudaPeekAtLastError();
     if (e != cudaSuccess) (void)cudaGetLastError();
     return e;
 }
@@ -1594,20 +1622,19 @@ extern "C" lmosem_status lmosem_osem_subiter_noalloc(const float* d_rows, int64_
     // an error left by earlier work stays the caller's to read: run nothing
     if (cudaPeekAtLastError() != cudaSuccess) return LMOSEM_ECUDA;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const NoAllocDevice* dev = nullptr;
-    if (noalloc_device(&dev) != cudaSuccess) return LMOSEM_ECUDA;
+    float* scratch = nullptr;
+    if (noalloc_scratch(&scratch) != cudaSuccess) return LMOSEM_ECUDA;
 
     // same column-vector shape as the context path (FP32 rows, 4 per vector)
     const int64_t nvec = ld / 4;
-    int w = kNoAllocKernels - 1;
-    for (int k = 0; k < kNoAllocKernels; ++k)
-        if ((nvec + kNoAllocWidths[k] - 1) / kNoAllocWidths[k] <= kMaxPassThreads) {
-            w = k;
+    const int opts[] = {1, 2, 3, 4, 6, kNoAllocMaxVpt};
+    int vpt = kNoAllocMaxVpt;
+    for (int v : opts)
+        if ((nvec + v - 1) / v <= kMaxPassThreads) {
+            vpt = v;
             break;
         }
-    const int vpt = kNoAllocWidths[w];
     const int nt = (int)(((nvec + vpt - 1) / vpt + 31) / 32 * 32);
-    const int sms = dev->sms, per_sm = dev->per_sm[w][nt / 32];
     PassArgs A;
     A.model = d_rows;
     A.ld_bytes = ld * 4;
@@ -1620,24 +1647,23 @@ extern "C" lmosem_status lmosem_osem_subiter_noalloc(const float* d_rows, int64_
     A.weight = nullptr;
     A.n_sup = n_support;
     A.log_T = 0.0;
-    A.bpart = dev->scratch;
+    A.bpart = scratch;
     A.llpart = nullptr;
     A.prefetch = 0;
     int grid = 0;
     cudaError_t e;
     switch (vpt) {
-        case 1: e = noalloc_pass<1>(A, n_rows, nt, sms, per_sm, s, &grid); break;
-        case 2: e = noalloc_pass<2>(A, n_rows, nt, sms, per_sm, s, &grid); break;
-        case 3: e = noalloc_pass<3>(A, n_rows, nt, sms, per_sm, s, &grid); break;
-        case 4: e = noalloc_pass<4>(A, n_rows, nt, sms, per_sm, s, &grid); break;
-        case 6: e = noalloc_pass<6>(A, n_rows, nt, sms, per_sm, s, &grid); break;
-        default: e = noalloc_pass<kNoAllocMaxVpt>(A, n_rows, nt, sms, per_sm, s, &grid); break;
+        case 1: e = noalloc_pass<1>(A, n_rows, nt, s, &grid); break;
+        case 2: e = noalloc_pass<2>(A, n_rows, nt, s, &grid); break;
+        case 3: e = noalloc_pass<3>(A, n_rows, nt, s, &grid); break;
+        case 4: e = noalloc_pass<4>(A, n_rows, nt, s, &grid); break;
+        case 6: e = noalloc_pass<6>(A, n_rows, nt, s, &grid); break;
+        default: e = noalloc_pass<kNoAllocMaxVpt>(A, n_rows, nt, s, &grid); break;
     }
     if (e != cudaSuccess) return LMOSEM_ECUDA;
-    // 193 CTAs of 8 pixels at 1,540 columns; 49 CTAs of 32 took 7 us instead of 5
-    e = launch_pdl(k_update_px, dim3((n_support + kUpdPix - 1) / kUpdPix), dim3(kUpdPix * kUpdGroups), 0, s,
-                   (const float*)dev->scratch, grid, (int)n_support, d_f, d_sens_i, acq_time, (const int*)nullptr);
-    if (e != cudaSuccess) {
+    k_update<<<(n_support + 31) / 32, 256, 0, s>>>(scratch, grid, n_support, d_f, d_sens_i, acq_time,
+                                                   nullptr);
+    if (cudaPeekAtLastError() != cudaSuccess) {
         (void)cudaGetLastError();
         return LMOSEM_ECUDA;
     }
