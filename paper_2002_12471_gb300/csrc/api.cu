@@ -234,9 +234,13 @@ lmosem_status build_model_common(lmosem_ctx* c, const int32_t* d_angle, const fl
     }
     bool grid = false;
     int64_t n_outside = 0;
-    if ((st = grid_plan(c, n_events, &grid)) ||
-        (st = sort_events(c, d_angle, d_u_mm, d_e_kev, n_events, n_subsets, h_offsets, n_real,
-                          grid ? &n_outside : nullptr))) {
+    st = grid_plan(c, n_events, &grid);
+    if (st == LMOSEM_ENOMEM) {  // no room for its tables: the path sum
+        st = LMOSEM_OK;
+        grid = false;
+    }
+    if (st || (st = sort_events(c, d_angle, d_u_mm, d_e_kev, n_events, n_subsets, h_offsets, n_real,
+                                grid ? &n_outside : nullptr))) {
         free_model(c);
         return st;
     }
@@ -780,8 +784,10 @@ lmosem_status lmosem_reconstruct(lmosem_ctx* c, const int32_t* h_angle, const fl
     LMOSEM_CK(c, cudaMemcpyAsync(d_a, h_angle, n * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
     LMOSEM_CK(c, cudaMemcpyAsync(d_u, h_u_mm, n * sizeof(float), cudaMemcpyHostToDevice, c->stream));
     LMOSEM_CK(c, cudaMemcpyAsync(d_e, h_e_kev, n * sizeof(float), cudaMemcpyHostToDevice, c->stream));
-    if ((st = lmosem_sensitivity(c, n_subsets, nullptr)) ||
-        (st = lmosem_build_model(c, d_a, d_u, d_e, n_events, n_subsets, fmt)) ||
+    if (grid_plan(c, n_events, &c->grid_expected)) c->grid_expected = false;
+    st = lmosem_sensitivity(c, n_subsets, nullptr);
+    c->grid_expected = false;
+    if (st || (st = lmosem_build_model(c, d_a, d_u, d_e, n_events, n_subsets, fmt)) ||
         (st = lmosem_init_image(c, T, d_f)) || (st = lmosem_iterate(c, n_iters, T, d_f, nullptr)) ||
         (h_loglik && (st = lmosem_loglik(c, T, d_f, d_ll)))) {
         drop_graph(c);

@@ -131,6 +131,7 @@ struct lmosem_ctx {
     bool terms_pending = false;   // the last build used the grid: the terms are counted when asked for
     lmosem::GridPlan grid;
     bool use_grid = false;        // the model's exact rows come from the grid
+    bool grid_expected = false;   // the next build's will: the sensitivity leaves the scatter planes out
     int* d_status = nullptr;      // [0] = 1 after a bounded device wait ran out
     long long wait_budget = 2000000000LL;  // clock cycles per bounded wait
     int pass_variant = 0;         // 0 auto, 1 register pipeline, 2 bulk-copy ring, 3 cp.async ring,
@@ -350,7 +351,7 @@ lmosem_status compute_sensitivity(lmosem_ctx* c, int n_subsets);  // sens.cu
 // model.cu: every angle's scatter-weight planes into d_wtab_all and, in the
 // same pass, the per-angle sensitivities (arithmetic of the sensitivity
 // kernel: FP32 terms, FP64 every 32 terms); false from wtab_all_fits when
-// the planes of all angles exceed the table budget
+// the planes of all angles exceed the table budget or are not wanted
 bool wtab_all_fits(const lmosem_ctx* c);
 lmosem_status wtab_all_with_sens(lmosem_ctx* c, double* sens_angle, float w_const_sens, float de0);
 lmosem_status run_iterations(lmosem_ctx* c, int n_iters, double T, float* d_f, double* d_ll);

@@ -1211,14 +1211,15 @@ lmosem_status hull_reset(lmosem_ctx* c, const WTabArgs& W, int n) {
 
 }  // namespace
 
-// Planes of every angle in the sensitivity's pass, while they are small enough.
-// At 50 x 50 (1.0 GB, 37k events) the whole reconstruction took 4.1 ms with
-// the fused pass and 4.3 without; at 64 x 64 (3.7 GB) the fused pass took 2.09 ms
-// and the planes' allocation 2.7 ms of host time, against 1.09 ms for the
-// sensitivity alone and 1.1 ms for k_wtable, which the grid form does without.
+// Planes of every angle in the sensitivity's pass, unless the build that
+// follows is known to form its rows on the grid, which does without them: at
+// 64 x 64 (3.7 GB) the fused pass takes 2.09 ms and the planes' allocation 2.7 ms
+// of host time, the sensitivity alone 1.09 ms.  For the path sum and the binned
+// rows the fused pass is the better one (71 x 71, 42 angles, 6,756 events: the
+// whole reconstruction 4.83 ms, 5.07 with sensitivity and planes apart).
 bool wtab_all_fits(const lmosem_ctx* c) {
     const int64_t bytes = (int64_t)c->n_angles * wtab_angle_floats(c) * (int64_t)sizeof(float);
-    return bytes <= std::min<int64_t>(c->table_budget, int64_t(1280) << 20) && c->n_scat <= 32 * 128;
+    return !c->grid_expected && bytes <= c->table_budget && c->n_scat <= 32 * 128;
 }
 
 lmosem_status wtab_all_with_sens(lmosem_ctx* c, double* sens_angle, float w_const_sens, float de0) {
