@@ -93,8 +93,9 @@ typedef struct {
      * their CUDA-graph replay on non-default streams and are not timed. */
     int32_t profile;
     /* Clock-cycle budget of every bounded device wait (the mbarrier waits of
-     * the TMA-ring OSEM pass, the tensor-core surrogate and the batch
-     * scheduler's work queue; the path sum and the other passes wait only at
+     * the TMA-ring OSEM pass, the tensor-core surrogate, the batch scheduler's
+     * work queue and the scatter sum that the model build of a large event
+     * list forms on a grid; the path sum and the other passes wait only at
      * CTA barriers); 0 selects 2e9 (about one second).
      * A wait that runs out abandons its kernel and the call returns
      * LMOSEM_ETIMEOUT; the context stays usable.  Tests set a tiny budget
@@ -216,9 +217,12 @@ lmosem_status lmosem_sensitivity(lmosem_ctx* ctx, int32_t n_subsets, double* d_s
  * in mm, energy in keV).  The context sorts them by (subset, angle, energy
  * class, u), the class splitting at E0 (1 - fwhm_frac_e0 / 2), and keeps
  * the sorted copy; the caller's arrays are not modified and may be
- * freed on return.  Synchronises the stream (input check).
+ * freed on return.  Synchronises the stream (input check; a large event list,
+ * whose scatter sum is formed on a grid, also at the end, for the status of
+ * its bounded waits).
  * EINVAL: n_events < 1 or >= 2^31, n_subsets not in [1, n_angles], an angle
  * outside [0, n_angles), |u| > extent/2, E outside [e_lo, e_hi], NaN.
+ * ETIMEOUT: a bounded device wait ran out; no model is kept.
  * ENOMEM: the model does not fit.  Any earlier model is released first. */
 lmosem_status lmosem_build_model(lmosem_ctx* ctx, const int32_t* d_angle, const float* d_u_mm,
                                  const float* d_e_kev, int64_t n_events, int32_t n_subsets,

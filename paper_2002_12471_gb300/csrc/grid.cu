@@ -50,7 +50,6 @@ static_assert(kSub == 64, "two ballots");
 static_assert(kEpi == 16 && kWin % kEpi == 0 && kWin % 16 == 0, "whole steps");
 constexpr int kEGroup = 8;                  // energy nodes per CTA: 4 lane groups x 2
 constexpr int kNTile = 32;                  // support pixels per CTA
-constexpr long long kGridBudget = 2000000000LL;  // clock cycles per bounded wait (about a second)
 
 // ---------------------------------------------------------------- plan
 
@@ -1289,7 +1288,7 @@ lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& s
         S.out_scale = (float)exp2(-(double)G.log_g - (double)G.log_u);
         S.T = T;
         S.status = c->d_status;
-        S.budget = kGridBudget;
+        S.budget = c->wait_budget;
         LMOSEM_PROF_BEGIN(c);
         k_grid_sum<<<(unsigned)(na * S.n_nt * (G.ne / kEGroup)), kGridThreads, kSmBytes, c->stream>>>(S);
         LMOSEM_LAUNCHED(c, LMOSEM_K_PATHSUM);
