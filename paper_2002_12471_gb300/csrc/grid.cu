@@ -1026,8 +1026,10 @@ CellArgs cell_args(const lmosem_ctx* c, const int32_t* a, const float* u, const 
 lmosem_status grid_plan(lmosem_ctx* c, int64_t n, bool* use) {
     *use = false;
     if (n < (int64_t)64 * c->n_angles || c->n_scat < 2 * kSub || c->n_scat > 16384) return LMOSEM_OK;
-    // narrower cuts than the default leave steps in S_n
-    if (c->k_sigma < 6.0f || (c->e_sigma > 0.0f && c->e_sigma < 6.0f)) return LMOSEM_OK;
+    // Only for the default cuts.  Narrower ones leave steps in S_n; a wider position cut asks for terms beyond
+    // kFarSigma of the widest response, which the window of nodes does not hold; no energy cut asks for the exact
+    // sum.  (A wider energy cut drops fewer terms than the default, and the grid drops none by energy.)
+    if (c->k_sigma != 6.0f || c->e_sigma < 6.0f) return LMOSEM_OK;
     GridPlan& G = c->grid;
     if (G.state == 0) {
         G.state = 1;  // not usable unless set below
@@ -1042,7 +1044,7 @@ lmosem_status grid_plan(lmosem_ctx* c, int64_t n, bool* use) {
         const double s_min = (c->fwhm0 + c->fwhm_slope * (c->radius - rmax)) * f2s;
         const double s_max = (c->fwhm0 + c->fwhm_slope * (c->radius + rmax)) * f2s;
         const double s_lat = (c->fwhm0 + c->fwhm_slope * c->radius) * f2s;  // of the outermost pixels
-        const double half = 0.5 * c->n_bins * c->bin_mm, cut = std::min((double)c->k_sigma, kFarSigma) * s_max;
+        const double half = 0.5 * c->n_bins * c->bin_mm, cut = kFarSigma * s_max;
         // The window of nodes has to hold the widest response.  A scatter pixel whose k_sigma cut is longer than
         // kFarSigma of the widest (the last few centimetres of depth) is cut there instead: what is left out is
         // below 4e-8 of its response's mass.  The pixels that bound the object sideways keep their whole cut.
