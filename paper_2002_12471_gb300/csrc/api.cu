@@ -244,8 +244,7 @@ lmosem_status build_model_common(lmosem_ctx* c, const int32_t* d_angle, const fl
         free_model(c);
         return st;
     }
-    // rows outside the grid's region cost about 30 times a path-sum row
-    c->use_grid = grid && n_outside <= n_events / 128;
+    c->use_grid = grid && n_outside <= c->grid.max_direct;  // their rows are summed directly
     if ((st = sur ? build_checked_surrogate(c) : build_model_rows(c))) {
         free_model(c);
         return st;

@@ -1022,7 +1022,9 @@ CellArgs cell_args(const lmosem_ctx* c, const int32_t* a, const float* u, const 
 //  * the path sum: 5.5e12 terms per second, 0.8 of the position strip's terms
 //    being kept by the energy cut.
 // They meet near 500 events per angle at 128 x 128 (6,000 pixels) and near
-// 1,000 at 64 x 64 (1,540); the grid has to win by a tenth.
+// 1,000 at 64 x 64 (1,540); the grid has to win by a tenth, with every row that
+// is summed directly (k_grid_direct) counted as 30 of the path sum's: at most
+// max_direct of them.
 lmosem_status grid_plan(lmosem_ctx* c, int64_t n, bool* use) {
     *use = false;
     if (n < (int64_t)64 * c->n_angles || c->n_scat < 2 * kSub || c->n_scat > 16384) return LMOSEM_OK;
@@ -1088,6 +1090,7 @@ lmosem_status grid_plan(lmosem_ctx* c, int64_t n, bool* use) {
                                          tiles * G.n_sub * 25e-9) + n * tiles * 400.0 / per_s + 60e-6;
     const double t_path = n * (0.8 * G.strip * c->n_scat * c->n_sup) / 5.5e12;
     if (!(t_grid < 0.9 * t_path)) return LMOSEM_OK;
+    G.max_direct = (int64_t)((0.9 - t_grid / t_path) * n / 30.0);
     *use = true;
     if (G.state == 3) return LMOSEM_OK;
     const double kappa = kappa_of(c);

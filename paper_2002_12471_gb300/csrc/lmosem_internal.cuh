@@ -39,6 +39,7 @@ struct GridPlan {
     double edge = 0, e_min = 0, e_max = 0;  // events beyond are summed directly
     int max_sub = 0, n_sub = 0;  // subgroups per angle at most, and about
     double strip = 0;            // share of the scatter pixels within an event's position cut
+    int64_t max_direct = 0;      // rows of the last planned list that may be summed directly
     float log_g = 0, log_u = 0;  // log2 of the operands' scales
     int32_t* d_slot_m = nullptr; // [a][subgroup][64]: scatter pixel or -1
     int32_t* d_i0 = nullptr;     // [a][subgroup]: first node
