@@ -228,8 +228,11 @@ lmosem_status lmosem_sensitivity(lmosem_ctx* ctx, int32_t n_subsets, double* d_s
  * The scatter sum is formed path by path (FP32 terms and sums), or, when that
  * is cheaper and k_sigma and e_sigma allow it, on a grid of detector positions
  * and energies per angle and interpolated at the events: lists of some hundred
- * events per angle and more.  Both agree with the exact sum within 6e-6 of a
- * row's largest entry (measured; about 4e-7 in relative L2 over the rows).
+ * events per angle and more.  Rows there that are small against the grid values
+ * around them (energies or positions that hardly a path reaches) are summed path
+ * by path, and so is the whole list when they are many.  Both forms agree with
+ * the exact sum within 6e-6 of a row's largest entry (measured; about 4e-7 in
+ * relative L2 over the rows).
  * Synchronises the stream (input check; a large event list,
  * whose scatter sum is formed on a grid, also at the end, for the status of
  * its bounded waits).

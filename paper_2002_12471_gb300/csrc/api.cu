@@ -244,7 +244,9 @@ lmosem_status build_model_common(lmosem_ctx* c, const int32_t* d_angle, const fl
         free_model(c);
         return st;
     }
-    c->use_grid = grid && n_outside <= c->grid.max_direct;  // their rows are summed directly
+    // the rows outside the grid's region are among those summed directly
+    c->use_grid = grid && n_outside <= c->grid.max_direct;
+    c->grid_max_direct = c->grid.max_direct - n_outside;
     if ((st = sur ? build_checked_surrogate(c) : build_model_rows(c))) {
         free_model(c);
         return st;
@@ -440,6 +442,7 @@ lmosem_status lmosem_create(const lmosem_object* obj, const lmosem_geometry* geo
         bool sup = obj->h_support ? obj->h_support[p] != 0 : v > 0.0;
         if (sup) c->h_sup.push_back(p);
         if (v > 0.0) c->h_scat.push_back(p);
+        if (v > 0.0 && !sup) c->partial_support = true;
         if (sup || v > 0.0) {
             double x = (p % c->nx + 0.5 - 0.5 * c->nx) * c->dpx;
             double y = (p / c->nx + 0.5 - 0.5 * c->ny) * c->dpx;

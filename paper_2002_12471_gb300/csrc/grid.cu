@@ -929,11 +929,120 @@ __global__ void __launch_bounds__(128) k_grid_rows(RowArgs A) {
     }
 }
 
-// Rows of the events outside the grid's region, summed path by path.
+// The interpolation's error is absolute: about 4e-7 of the largest of the grid
+// values that it combines.  Where S_n falls steeply for every n (energies above
+// every Compton energy that reaches a position, positions that no scatter pixel
+// looks at) and no primary covers it, that is no longer small against the row:
+// for a unit Gaussian 1.3e-6 of the value 2 sigma out, 5e-6 at 2.5, 1.3e-5 at 3,
+// 3e-4 at 4.  Such rows are summed path by path.  An event's row is taken to be
+// steep when its largest value (of S_n over the support, interpolated in the
+// logarithm, or of the primary) is below 1 / kSteep of the largest S_n 4 nodes
+// away along one of the axes (1 sigma in x, 1.7 of the narrowest sigma in u):
+// from 2.6 sigma on in x, and in u from 2.1 sigma of the narrowest response on
+// and 3.5 of one twice as wide, which the grid resolves better.
+constexpr float kSteepLog2 = 3.0f;
+constexpr int kTopStep = 4;      // nodes between those where the largest S_n is taken
+
+// log2 of the largest S_n over the support at every kTopStep-th node of either
+// axis, 4 warps per node: a sixteenth of T is read, which bounds it.  (Taken in
+// the sum's epilogue it cost 1.5 to 3% of the sum.)  Also keeps the length of
+// the list of directly summed rows before this group.
+__global__ void __launch_bounds__(128) k_grid_top(const float* __restrict__ T, int ne, int nu, int ld,
+                                                  float* __restrict__ top, const int32_t* n_list, int32_t* n_list0) {
+    __shared__ float sh[4];
+    if (blockIdx.x + blockIdx.y + blockIdx.z == 0 && threadIdx.x == 0) *n_list0 = *n_list;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_full = ld / kTCols, n_tiles = (ld + kTCols - 1) / kTCols;
+    const float* t = T + (((size_t)blockIdx.z * n_tiles * ne + kTopStep * blockIdx.y) * nu + kTopStep * blockIdx.x) * kTCols +
+                     4 * lane;
+    float mx = 0.0f;
+    auto take = [&](int k) {
+        const float4 v = *reinterpret_cast<const float4*>(t + (size_t)k * ne * nu * kTCols);
+        mx = fmaxf(fmaxf(mx, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
+    };
+#pragma unroll 4
+    for (int k = warp; k < n_full; k += 4) take(k);
+    if (warp == n_full % 4 && n_full * kTCols + 4 * lane < ld) take(n_full);  // (columns past ld are not written)
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) sh[warp] = mx;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        top[((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] =
+            __log2f(fmaxf(fmaxf(fmaxf(sh[0], sh[1]), fmaxf(sh[2], sh[3])), 1e-37f));
+}
+
+struct TailArgs {
+    const GridEvent* ev;
+    const int32_t* off;
+    int cell0, cell1;            // blocks of the group
+    int per_slot, s0;            // per_slot: blocks of cells
+    int nx, nm;                  // nodes of top
+    const float* top;            // [angle of the group][nx][nm]
+    const float* pmax;           // [slot][nm]: log2 of the largest primary, without its energy factor
+    float u_lo, inv_hu, x_lo, inv_hx, inv_kappa;
+    float e0, sE0, lE0;
+    int max_list;
+    int32_t* list;               // places in ev of the rows to be summed directly
+    int32_t* n_list;             // rows found so far, those of earlier groups included
+};
+__global__ void __launch_bounds__(256) k_grid_tails(TailArgs A) {
+    const int p = A.off[A.cell0] + blockIdx.x * 256 + threadIdx.x;
+    if (p >= A.off[A.cell1]) return;
+    const float4 h = *reinterpret_cast<const float4*>(A.ev + p);
+    const int s = (__float_as_int(h.y) >> 2) / A.per_slot;
+    // place among the nodes, and among those of top
+    const float iu = fmaxf((h.z - A.u_lo) * A.inv_hu, 0.0f) + (kPU / 2 - 1);
+    const float ix = fmaxf((2.0f * sqrtf(h.w * A.inv_kappa) - A.x_lo) * A.inv_hx, 0.0f) + (kPE / 2 - 1);
+    const int ju = (int)(iu / kTopStep), jx = (int)(ix / kTopStep);
+    const float fu = iu / kTopStep - ju, fx = ix / kTopStep - jx;
+    const float* t = A.top + (size_t)(s - A.s0) * A.nx * A.nm;
+    auto at = [&](int dx, int du) {  // dx, du nodes of top from the event
+        const int x0 = min(max(jx + dx, 0), A.nx - 1), x1 = min(max(jx + dx + 1, 0), A.nx - 1);
+        const int u0 = min(max(ju + du, 0), A.nm - 1), u1 = min(max(ju + du + 1, 0), A.nm - 1);
+        const float a = t[x0 * A.nm + u0], b = t[x0 * A.nm + u1], c = t[x1 * A.nm + u0], d = t[x1 * A.nm + u1];
+        const float lo = fmaf(fu, b - a, a), hi = fmaf(fu, d - c, c);
+        return fmaf(fx, hi - lo, lo);
+    };
+    const float around = fmaxf(fmaxf(at(-1, 0), at(1, 0)), fmaxf(at(0, -1), at(0, 1)));
+    const float te = (h.w - A.e0) * A.sE0;
+    const float* pm = A.pmax + (size_t)s * A.nm;
+    const float p0 = pm[min(ju, A.nm - 1)], p1 = pm[min(ju + 1, A.nm - 1)];
+    const float row = fmaxf(at(0, 0), fmaf(fu, p1 - p0, p0) + fmaf(-te, te, A.lE0));
+    if (row + kSteepLog2 >= around) return;
+    const int k = atomicAdd(A.n_list, 1);
+    if (k < A.max_list) A.list[k] = p;
+}
+// log2 of the largest primary over the support at every kTopStep-th position
+// node, without the energy factor
+__global__ void __launch_bounds__(128) k_grid_prim(const float4* __restrict__ ppar, const int32_t* __restrict__ slot_angle,
+                                                   int ld_w, int n_sup, double u_node0, double step,
+                                                   float* __restrict__ pmax) {
+    __shared__ float sh[4];
+    const float4* pp = ppar + (size_t)slot_angle[blockIdx.y] * ld_w;
+    const float u = (float)(u_node0 + blockIdx.x * step);
+    float mx = -INFINITY;
+    for (int n = threadIdx.x; n < n_sup; n += 128) {
+        const float4 q = __ldg(pp + n);
+        const float t = (u - q.x) * q.y;
+        mx = fmaxf(mx, fmaf(-t, t, q.z));
+    }
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        pmax[(size_t)blockIdx.y * gridDim.x + blockIdx.x] =
+            fmaxf(fmaxf(fmaxf(sh[0], sh[1]), fmaxf(sh[2], sh[3])), -1000.0f);
+}
+
+// Rows of the events outside the grid's region and of the steep rows, summed
+// path by path, nothing shared between them.
 struct DirectArgs {
     const GridEvent* ev;
     const int32_t* off;
     int key0, key1;              // keys of the group's events outside the grid
+    const int32_t* list;         // places in ev of the steep rows:
+    const int32_t* list0;        // the group's first one
+    const int32_t* n_list;       // all found so far; none is summed here once there are more than max_list
+    int max_list, per_slot;      // per_slot: blocks of cells
     int ncells, s0;
     const int32_t* slot_angle;
     const float4* planes;
@@ -949,30 +1058,59 @@ struct DirectArgs {
     float* out;
     int64_t ld_out, row_base;
 };
+// One CTA per (128 columns, row): 128 scatter pixels at a time, those within
+// their cut listed in shared memory, so that the table values of several of
+// them are in flight (a group with one row at 64 x 64: 40 us, about 350 with the
+// test and the loads of one pixel after the other).
 __global__ void __launch_bounds__(128) k_grid_direct(DirectArgs A) {
-    const int n = blockIdx.x * 128 + threadIdx.x;
-    if (n >= A.ld) return;
-    const bool real = n < A.n_sup;
-    for (int p = A.off[A.key0] + blockIdx.y; p < A.off[A.key1]; p += gridDim.y) {
-        const GridEvent* ev = A.ev + p;
-        const int s = ev->cell - A.ncells, a = A.slot_angle[s];
+    __shared__ float2 near[128];  // (slot, U) of the pixels within their cut, in slot order
+    __shared__ int cnt[4];
+    const int n = blockIdx.x * 128 + threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool col = n < A.ld, real = n < A.n_sup;
+    const int out0 = A.off[A.key0], n_out = A.off[A.key1] - out0;
+    const int l0 = *A.list0, n_list = *A.n_list <= A.max_list ? *A.n_list - l0 : 0;
+    for (int j = blockIdx.y; j < n_out + n_list; j += gridDim.y) {
+        const GridEvent* ev = A.ev + (j < n_out ? out0 + j : A.list[l0 + j - n_out]);
+        const int s = j < n_out ? ev->cell - A.ncells : (ev->cell >> 2) / A.per_slot, a = A.slot_angle[s];
         const float u = ev->u, e = ev->e, E = e * A.cE2, El = fmaf(e, A.cE2, -E);
+        const int nc = col ? n : 0;  // threads past the row join the lists only
         const float4* pl =
-            A.planes + ((size_t)(s - A.s0) * (A.ld / kNTile) + n / kNTile) * (A.max_sub * kSub / 2) * kNTile + n % kNTile;
+            A.planes + ((size_t)(s - A.s0) * (A.ld / kNTile) + nc / kNTile) * (A.max_sub * kSub / 2) * kNTile + nc % kNTile;
         const int32_t* sm = A.slot_m + (size_t)a * A.max_sub * kSub;
+        const int n_slots = A.n_sub[a] * kSub;
         float acc = 0.0f;
-        for (int k = 0; k < A.n_sub[a] * kSub; ++k) {
-            const int m = __ldg(sm + k);
-            if (m < 0) continue;
-            const float4 q = __ldg(A.mpar + (size_t)a * A.n_scat + m);
-            const float d = u - q.x;
-            if (fabsf(d) > q.w) continue;
-            const float z = d * q.y;
-            const float U = ex2_approx(fmaf(-z, z, q.z));
-            const float* v = reinterpret_cast<const float*>(pl + (k >> 1) * kNTile);
-            const float e1 = v[k & 1], t = (E - e1 + El) * rsqrt_approx(e1);
-            acc = fmaf(U, ex2_approx(-fmaf(t, t, v[2 + (k & 1)])), acc);
+        for (int b = 0; b < n_slots; b += 128) {
+            const int k = b + threadIdx.x, m = k < n_slots ? __ldg(sm + k) : -1;
+            bool in = false;
+            float U = 0.0f;
+            if (m >= 0) {
+                const float4 q = __ldg(A.mpar + (size_t)a * A.n_scat + m);
+                const float d = u - q.x, z = d * q.y;
+                in = fabsf(d) <= q.w;
+                U = ex2_approx(fmaf(-z, z, q.z));
+            }
+            const unsigned bal = __ballot_sync(0xffffffffu, in);
+            __syncthreads();  // the last list is read
+            if (lane == 0) cnt[warp] = __popc(bal);
+            __syncthreads();
+            int first = 0, total = 0;
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                if (w < warp) first += cnt[w];
+                total += cnt[w];
+            }
+            if (in) near[first + __popc(bal & ((1u << lane) - 1u))] = make_float2(__int_as_float(k), U);
+            __syncthreads();
+#pragma unroll 8
+            for (int i = 0; i < total; ++i) {
+                const float2 q = near[i];
+                const int kk = __float_as_int(q.x);
+                const float* v = reinterpret_cast<const float*>(pl + (kk >> 1) * kNTile);
+                const float e1 = __ldg(v + (kk & 1)), w = __ldg(v + 2 + (kk & 1)), t = (E - e1 + El) * rsqrt_approx(e1);
+                acc = fmaf(q.y, ex2_approx(-fmaf(t, t, w)), acc);
+            }
         }
+        if (!col) continue;
         const float4 pp = A.ppar[(size_t)a * A.ld_w + n];
         const float te = (e - A.e0) * A.sE0, tu = (u - pp.x) * pp.y;
         const float prim = ex2_approx(fmaf(-tu, tu, pp.z + fmaf(-te, te, A.lE0)));
@@ -1024,7 +1162,8 @@ CellArgs cell_args(const lmosem_ctx* c, const int32_t* a, const float* u, const 
 // They meet near 500 events per angle at 128 x 128 (6,000 pixels) and near
 // 1,000 at 64 x 64 (1,540); the grid has to win by a tenth, with every row that
 // is summed directly (k_grid_direct) counted as 30 of the path sum's: at most
-// max_direct of them.
+// max_direct of them.  (Measured: 2.5 path-sum rows each for 1,000 at the edge of
+// the object at 64 x 64, more inside it, and the latency of one per group, 40 us.)
 lmosem_status grid_plan(lmosem_ctx* c, int64_t n, bool* use) {
     *use = false;
     if (n < (int64_t)64 * c->n_angles || c->n_scat < 2 * kSub || c->n_scat > 16384) return LMOSEM_OK;
@@ -1153,10 +1292,13 @@ lmosem_status grid_count_outside(lmosem_ctx* c, const int32_t* a, const float* u
     return LMOSEM_OK;
 }
 
-// FP32 rows of every sorted event (scaled forms: staged per group and handed
-// to `quantize`), angle group by angle group within the table budget.
-lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& slot_angle) {
+// Rows of every sorted event (scaled forms: staged as FP32 per group and
+// rounded), angle group by angle group within the table budget.  *done = false:
+// too many rows are steep (more than max_direct, or so many in the first group), and the path sum has to form them all.
+lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& slot_angle, int64_t max_direct,
+                                    bool* done) {
     const GridPlan& G = c->grid;
+    *done = false;
     lmosem_status st;
     if ((st = ensure_status(c))) return st;
     const int ns = (int)slot_angle.size(), ld = (int)c->ld_model;
@@ -1196,16 +1338,31 @@ lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& s
     const int64_t pairs = (int64_t)G.max_sub * kSub / 2;
     const int64_t plane_n = pairs * ld, t_n = (int64_t)G.ne * G.nu * ((ld + kTCols - 1) / kTCols * kTCols), u_n = (int64_t)G.max_sub * kUStage;
     const int64_t per_angle = plane_n * 16 + t_n * 4 + u_n;
+    const int top_x = (G.ne + kTopStep - 1) / kTopStep, top_u = (G.nu + kTopStep - 1) / kTopStep;
     // groups of at most 2 GiB: the pool maps fresh memory at about 0.7 ms per GB (64 x 64 with 200k events: build
     // 17.3 ms at 2 GiB, 18.2 at 1 GiB, 19.1 at 4 GiB)
-    const int gsz = (int)std::max<int64_t>(
+    int gsz = (int)std::max<int64_t>(
         1, std::min<int64_t>(ns, std::min<int64_t>(c->table_budget, int64_t(2) << 30) / per_angle));
+    // a support that leaves scatter pixels out is where steep rows are met: the first group shows it early
+    if (c->partial_support) gsz = std::min(gsz, std::max(1, ns / 8));
     float4* planes = nullptr;
     float* T = nullptr;
     unsigned char* ublob = nullptr;
+    const int max_list = (int)std::max<int64_t>(0, std::min<int64_t>(max_direct, J));
+    const int n_groups = (ns + gsz - 1) / gsz;
+    int32_t *list = nullptr, *n_list = nullptr;  // n_list[0]: rows found; [1 + gi]: before group gi
+    float *pmax = nullptr, *top = nullptr;
     if ((st = tmp.alloc(&planes, (size_t)gsz * plane_n)) || (st = tmp.alloc(&T, (size_t)gsz * t_n)) ||
-        (st = tmp.alloc(&ublob, (size_t)gsz * u_n)))
+        (st = tmp.alloc(&ublob, (size_t)gsz * u_n)) || (st = tmp.alloc(&top, (size_t)gsz * top_x * top_u)) ||
+        (st = tmp.alloc(&pmax, (size_t)ns * top_u)) || (st = tmp.alloc(&list, max_list)) ||
+        (st = tmp.alloc(&n_list, 1 + n_groups)))
         return st;
+    const double u_node0 = G.u_lo - (kPU / 2 - 1) * G.hu;
+    LMOSEM_CK(c, cudaMemsetAsync(n_list, 0, sizeof(int), c->stream));
+    LMOSEM_PROF_BEGIN(c);
+    k_grid_prim<<<dim3(top_u, ns), 128, 0, c->stream>>>(c->d_ppar, d_slot, c->ld_w, c->n_sup, u_node0, kTopStep * G.hu,
+                                                        pmax);
+    LMOSEM_LAUNCHED(c, LMOSEM_K_WTABLE);
     const bool scaled = c->fmt != LMOSEM_MODEL_FP32;
     std::vector<int64_t> g_rows, g_row0;
     for (int s0 = 0; s0 < ns; s0 += gsz) {
@@ -1224,6 +1381,9 @@ lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& s
         return st;
     LMOSEM_CK(c, cudaFuncSetAttribute(k_grid_sum, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmBytes));
     const float cE2 = (float)(1.4426950408889634 / (2.0 * kappa));
+    int64_t rows_done = 0;
+    bool looked = false;
+    int found = 0;
     for (int s0 = 0, gi = 0; s0 < ns; s0 += gsz, ++gi) {
         const int na = std::min(gsz, ns - s0);
         if (g_rows[gi] == 0) continue;
@@ -1240,7 +1400,7 @@ lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& s
         U.max_sub = G.max_sub;
         U.angle0 = c->angle0;
         U.dtheta = 2.0 * kPi / c->n_angles;
-        U.u_node0 = G.u_lo - (kPU / 2 - 1) * G.hu;
+        U.u_node0 = u_node0;
         U.hu = G.hu;
         U.cut = (float)G.cut;
         U.scale = G.log_u;
@@ -1323,11 +1483,44 @@ lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& s
         k_grid_rows<<<dim3((unsigned)((g_rows[gi] + kRowEvents - 1) / kRowEvents), (unsigned)((ld + 127) / 128)), 128, 0,
                       c->stream>>>(R);
         LMOSEM_LAUNCHED(c, LMOSEM_K_PATHSUM);
+        LMOSEM_PROF_BEGIN(c);
+        k_grid_top<<<dim3(top_u, top_x, na), 128, 0, c->stream>>>(T, G.ne, G.nu, ld, top, n_list, n_list + 1 + gi);
+        LMOSEM_LAUNCHED(c, LMOSEM_K_PATHSUM);
+        TailArgs Q;
+        Q.ev = ev;
+        Q.off = off;
+        Q.cell0 = R.cell0;
+        Q.cell1 = R.cell1;
+        Q.per_slot = nbx * nbu;
+        Q.s0 = s0;
+        Q.nx = top_x;
+        Q.nm = top_u;
+        Q.u_lo = (float)C.u_lo;
+        Q.inv_hu = (float)C.inv_hu;
+        Q.x_lo = (float)C.x_lo;
+        Q.inv_hx = (float)C.inv_hx;
+        Q.inv_kappa = (float)C.inv_kappa;
+        Q.top = top;
+        Q.pmax = pmax;
+        Q.e0 = R.e0;
+        Q.sE0 = R.sE0;
+        Q.lE0 = R.lE0;
+        Q.max_list = max_list;
+        Q.list = list;
+        Q.n_list = n_list;
+        LMOSEM_PROF_BEGIN(c);
+        k_grid_tails<<<(unsigned)((g_rows[gi] + 255) / 256), 256, 0, c->stream>>>(Q);
+        LMOSEM_LAUNCHED(c, LMOSEM_K_PATHSUM);
         DirectArgs D;
         D.ev = ev;
         D.off = off;
         D.key0 = (int)(ncells + s0);
         D.key1 = (int)(ncells + s0 + na);
+        D.list = list;
+        D.list0 = n_list + 1 + gi;
+        D.n_list = n_list;
+        D.max_list = max_list;
+        D.per_slot = nbx * nbu;
         D.ncells = (int)ncells;
         D.s0 = s0;
         D.slot_angle = d_slot;
@@ -1353,9 +1546,19 @@ lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& s
         k_grid_direct<<<dim3((unsigned)((ld + 127) / 128), 64), 128, 0, c->stream>>>(D);
         LMOSEM_LAUNCHED(c, LMOSEM_K_PATHSUM);
         if (scaled && (st = quantize_rows(c, g_rows[gi], g_row0[gi]))) return st;
+        rows_done += g_rows[gi];
+        if (rows_done < J && !looked) {  // the first group with events, if others follow
+            looked = true;
+            LMOSEM_CK(c, cudaMemcpyAsync(&found, n_list, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+            LMOSEM_CK(c, cudaStreamSynchronize(c->stream));
+            if (found > 32 && (double)found * J > (double)max_list * rows_done) break;
+        }
     }
     dev_free(c, &c->d_stage);
-    return take_status(c);  // a bounded wait that ran out; synchronises
+    LMOSEM_CK(c, cudaMemcpyAsync(&found, n_list, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    st = take_status(c);  // a bounded wait that ran out; synchronises
+    *done = rows_done == J && found <= max_list;
+    return st;
 }
 
 }  // namespace lmosem

@@ -69,6 +69,7 @@ struct lmosem_ctx {
     int n_sup = 0, n_scat = 0, ld_w = 0;  // ld_w: support padded to kTN
     std::vector<int32_t> h_sup, h_scat;
     double mu_max = 0;    // largest entry of the mu-map
+    bool partial_support = false;  // some scatter pixel is not in the support
     double kbar = 0;      // circle mean of the Klein-Nishina shape at E0
     double de0 = 0;       // energy-window mass of the photopeak
 
@@ -132,6 +133,7 @@ struct lmosem_ctx {
     bool terms_pending = false;   // the last build used the grid: the terms are counted when asked for
     lmosem::GridPlan grid;
     bool use_grid = false;        // the model's exact rows come from the grid
+    int64_t grid_max_direct = 0;  // steep rows of it that may be summed directly
     bool grid_expected = false;   // the next build's will: the sensitivity leaves the scatter planes out
     int* d_status = nullptr;      // [0] = 1 after a bounded device wait ran out
     long long wait_budget = 2000000000LL;  // clock cycles per bounded wait
@@ -339,7 +341,8 @@ lmosem_status grid_plan(lmosem_ctx* c, int64_t n_events, bool* use);
 void grid_free(lmosem_ctx* c);
 lmosem_status grid_count_outside(lmosem_ctx* c, const int32_t* a, const float* u, const float* e, int64_t n,
                                  int32_t* d_n);
-lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& slot_angle);
+lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& slot_angle, int64_t max_direct,
+                                    bool* done);
 // model.cu: staged FP32 rows (d_stage) to the scaled rows row0 ..; path terms of the current events
 lmosem_status quantize_rows(lmosem_ctx* c, int64_t rows, int64_t row0);
 lmosem_status count_terms(lmosem_ctx* c);

@@ -1276,12 +1276,13 @@ lmosem_status build_model_rows(lmosem_ctx* c) {
     const int ns = (int)slot_angle.size();
     if (c->use_grid && !c->scatter_only) {
         dev_free(c, &c->d_wtab_all);  // the grid has tables of its own
-        st = build_model_rows_grid(c, slot_angle);
-        if (st != LMOSEM_ENOMEM) {
+        bool done = false;
+        st = build_model_rows_grid(c, slot_angle, c->grid_max_direct, &done);
+        if (st != LMOSEM_ENOMEM && (st || done)) {
             c->terms_valid = c->terms_pending = st == LMOSEM_OK;
             return st;
         }
-        c->use_grid = false;  // its buffers do not fit beside the model: path by path
+        c->use_grid = false;  // its buffers do not fit beside the model, or too many rows are steep: path by path
     }
     c->terms_pending = false;
 
