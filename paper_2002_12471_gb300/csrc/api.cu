@@ -75,6 +75,13 @@ void free_model(lmosem_ctx* c) {
     dev_free(c, &c->d_stage);
     dev_free(c, &c->d_perm);
     dev_free(c, &c->d_rank);
+    if (c->terms_pending && !c->kept.u) {  // the count outlives the model: 8 bytes per event are kept for it
+        std::swap(c->kept.u, c->d_u_s);
+        std::swap(c->kept.e, c->d_e_s);
+        c->kept.n_real = c->n_real;
+        c->kept.row0 = c->h_angle_row0;
+        c->kept.cnt = c->h_angle_cnt;
+    }
     dev_free(c, &c->d_u_s);
     dev_free(c, &c->d_e_s);
     dev_free(c, &c->d_a_s);
@@ -89,7 +96,6 @@ void free_model(lmosem_ctx* c) {
     dev_free(c, &c->d_bpart_batch);
     dev_free(c, &c->d_weight);
     c->n_counts = 0.0;
-    if (c->terms_pending) c->terms_pending = c->terms_valid = false;  // their events are gone
     c->use_grid = false;
     c->bpart_batch_floats = 0;
     c->batch_model = false;
@@ -319,6 +325,7 @@ void lmosem_destroy(lmosem_ctx* c) {
     if (!c) return;
     cudaStreamSynchronize(c->stream);
     free_model(c);
+    drop_kept(c);
     dev_free(c, &c->d_wtab_all);
     dev_free(c, &c->d_mu);
     dev_free(c, &c->d_sup);
@@ -581,10 +588,6 @@ lmosem_status lmosem_build_model_binned(lmosem_ctx* c, const float* d_counts, in
         }
     }
     subset_row0[n_subsets] = r;
-    if (c->terms_pending) {  // the count of the last event list outlives it
-        lmosem_status st = count_terms(c);
-        if (st) return st;
-    }
     std::vector<int64_t> rank;  // ordinal of a positive bin in dense order -> row
     rank.reserve(n_rows);
     for (size_t q = 0; q < nbins; ++q)

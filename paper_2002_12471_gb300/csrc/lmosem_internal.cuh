@@ -27,6 +27,14 @@ constexpr int kTN = 128;
 constexpr int kMC = 32;
 constexpr int kBuildThreads = 256;
 
+// Sorted positions and energies of an event list, and where its angles' rows lie.
+struct TermEvents {
+    float* u = nullptr;
+    float* e = nullptr;
+    int n_real = 1;
+    std::vector<int64_t> row0, cnt;  // [r * n_angles + a]
+};
+
 // Grid of the scatter sum (grid.cu): its nodes, and per angle the scatter
 // pixels in subgroups of neighbouring positions.
 struct GridPlan {
@@ -131,6 +139,7 @@ struct lmosem_ctx {
     unsigned long long* d_terms = nullptr;  // path terms of the last model build (path-sum kernels)
     bool terms_valid = false;
     bool terms_pending = false;   // the last build used the grid: the terms are counted when asked for
+    lmosem::TermEvents kept;      // (u set) the pending count's events, no longer the model's
     lmosem::GridPlan grid;
     bool use_grid = false;        // the model's exact rows come from the grid
     int64_t grid_max_direct = 0;  // steep rows of it that may be summed directly
@@ -343,9 +352,10 @@ lmosem_status grid_count_outside(lmosem_ctx* c, const int32_t* a, const float* u
                                  int32_t* d_n);
 lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& slot_angle, int64_t max_direct,
                                     bool* done);
-// model.cu: staged FP32 rows (d_stage) to the scaled rows row0 ..; path terms of the current events
+// model.cu: staged FP32 rows (d_stage) to the scaled rows row0 ..; path terms of the pending count's events
 lmosem_status quantize_rows(lmosem_ctx* c, int64_t rows, int64_t row0);
 lmosem_status count_terms(lmosem_ctx* c);
+void drop_kept(lmosem_ctx* c);
 lmosem_status build_model_rows(lmosem_ctx* c);
 // binned rows: model of every (angle, position bin, energy bin) row of the
 // row map ([a][b][k] -> sorted row or -1) with energy bin edges e_edges

@@ -104,6 +104,8 @@ __device__ __forceinline__ void hull_fold(uint2* dst, uint2 v) {
 // planes (s, b, -lw) of the scatter path (n, m) at the angles of the group's
 // slots: one thread per (n, m) walks the slots, so the angle-free inputs
 // (the pair integral, the scatter pixel) are read once for all of them
+// (PLANES = false: the energy hulls alone, for counting terms)
+template <bool PLANES = true>
 __global__ void k_wtable(WTabArgs A, int n_slots) {
     int n = blockIdx.x * blockDim.x + threadIdx.x;
     int k = blockIdx.y;
@@ -114,7 +116,7 @@ __global__ void k_wtable(WTabArgs A, int n_slots) {
     const int pn = real ? A.sup[n] : 0;
     const float4 gm = __ldg(A.scat_geo + k);
     const int pm = __float_as_int(gm.w);
-    const float lpair = real ? A.l_pair[(size_t)k * A.n_sup + n] : 0.0f;
+    const float lpair = PLANES && real ? A.l_pair[(size_t)k * A.n_sup + n] : 0.0f;
     const float xn = pixel_x(pn, A.nx, A.dpx), yn = pixel_y(pn, A.nx, A.ny, A.dpx);
     for (int g = 0; g < n_slots; ++g) {
         float s = 0.0f, b = 0.0f, nlw = INFINITY;
@@ -126,19 +128,23 @@ __global__ void k_wtable(WTabArgs A, int n_slots) {
                 float P, kt;
                 compton(cpsi, A.eps0, A.inv_kbar, &P, &kt);
                 float e1 = A.e0 * P;
-                float ratio = compton_lookup(A.compton, cpsi).x;
-                float att = fmaf(ratio, A.l_edge[(size_t)a * A.npix + pm], lpair);
                 float ri = rsqrtf(e1);
-                nlw = fmaf(att, kLog2e, -__log2f(A.w_const * gm.z * kt * rinv * ri));
-                s = A.cE * ri;
-                b = -e1 * s;
+                if (PLANES) {
+                    float ratio = compton_lookup(A.compton, cpsi).x;
+                    float att = fmaf(ratio, A.l_edge[(size_t)a * A.npix + pm], lpair);
+                    nlw = fmaf(att, kLog2e, -__log2f(A.w_const * gm.z * kt * rinv * ri));
+                    s = A.cE * ri;
+                    b = -e1 * s;
+                }
                 hb = hull_bits(e1, ri, A.hK);
             }
         }
-        float* out = base + (size_t)g * 3 * plane;
-        out[0] = s;
-        out[plane] = b;
-        out[2 * plane] = nlw;
+        if (PLANES) {
+            float* out = base + (size_t)g * 3 * plane;
+            out[0] = s;
+            out[plane] = b;
+            out[2 * plane] = nlw;
+        }
         // whole warps share k and a 32-column slice of one tile (ld_w is a
         // multiple of kTN and the grid's surplus threads are whole warps)
         hull_fold(A.hull + ((size_t)g * A.n_ptiles + n / kTN) * A.n_scat + k, hb);
@@ -1279,12 +1285,14 @@ lmosem_status build_model_rows(lmosem_ctx* c) {
         bool done = false;
         st = build_model_rows_grid(c, slot_angle, c->grid_max_direct, &done);
         if (st != LMOSEM_ENOMEM && (st || done)) {
+            drop_kept(c);
             c->terms_valid = c->terms_pending = st == LMOSEM_OK;
             return st;
         }
         c->use_grid = false;  // its buffers do not fit beside the model, or too many rows are steep: path by path
     }
     c->terms_pending = false;
+    drop_kept(c);
 
     // angle groups bounded by the scatter-table budget (three FP32 planes);
     // one group indexed by angle when the sensitivity pass left every
@@ -1386,7 +1394,7 @@ lmosem_status build_model_rows(lmosem_ctx* c) {
             WTabArgs W = wtab_args(c, c->d_wtab, gsz, d_slot_angle, s0);
             if ((st = hull_reset(c, W, s1 - s0))) return st;
             LMOSEM_PROF_BEGIN(c);
-            k_wtable<<<dim3((c->ld_w + 255) / 256, c->n_scat), 256, 0, c->stream>>>(W, s1 - s0);
+            k_wtable<true><<<dim3((c->ld_w + 255) / 256, c->n_scat), 256, 0, c->stream>>>(W, s1 - s0);
             LMOSEM_LAUNCHED(c, LMOSEM_K_WTABLE);
         }
 
@@ -1548,32 +1556,44 @@ __global__ void __launch_bounds__(256) k_count_terms(TermArgs A) {
 
 }  // namespace
 
-// Path terms of the current events (rows built on the grid are no sums of
-// terms; the count stays that of the sum they evaluate)
+void drop_kept(lmosem_ctx* c) {
+    dev_free(c, &c->kept.u);
+    dev_free(c, &c->kept.e);
+}
+
+// Path terms of the events of the last build on the grid, whose rows are no sums
+// of terms: the count stays that of the sum they evaluate.  Their events are the
+// model's, or those kept aside when the model was released or replaced.
 lmosem_status count_terms(lmosem_ctx* c) {
     lmosem_status st;
+    const bool kept = c->kept.u != nullptr;
+    const float *u = kept ? c->kept.u : c->d_u_s, *e = kept ? c->kept.e : c->d_e_s;
+    const std::vector<int64_t>&row0 = kept ? c->kept.row0 : c->h_angle_row0, &cnt = kept ? c->kept.cnt : c->h_angle_cnt;
+    const int n_real = kept ? c->kept.n_real : c->n_real;
     if (!c->d_terms && (st = dev_alloc(c, &c->d_terms, 1))) return st;
     LMOSEM_CK(c, cudaMemsetAsync(c->d_terms, 0, sizeof(unsigned long long), c->stream));
     const int na = c->n_angles;
+    // the energy hulls of a group of angles: at most 64 MB, 2.3 MB per angle at 128 x 128
+    const int64_t hull_angle = (int64_t)c->n_scat * (c->ld_w / kTN);
     const int gsz = (int)std::max<int64_t>(
-        1, std::min<int64_t>(na, c->table_budget / (wtab_angle_floats(c) * (int64_t)sizeof(float))));
+        1, std::min<int64_t>(na, std::min<int64_t>(c->table_budget, int64_t(64) << 20) / (hull_angle * (int64_t)sizeof(uint2))));
     std::vector<int32_t> ident(na);
     std::vector<int64_t> ent, first(1, 0);
     for (int a = 0; a < na; ++a) ident[a] = a;
     for (int a0 = 0; a0 < na; a0 += gsz) {
         for (int a = a0; a < std::min(na, a0 + gsz); ++a)
-            for (int r = 0; r < c->n_real; ++r) {
+            for (int r = 0; r < n_real; ++r) {
                 const size_t k = (size_t)r * na + a;
-                if (c->h_angle_cnt[k] > 0) ent.insert(ent.end(), {a, a - a0, c->h_angle_row0[k], c->h_angle_cnt[k]});
+                if (cnt[k] > 0) ent.insert(ent.end(), {a, a - a0, row0[k], cnt[k]});
             }
         first.push_back((int64_t)ent.size() / 4);
     }
     int32_t* d_ang = nullptr;
     int64_t* d_ent = nullptr;
-    float* wtab = nullptr;
+    uint2* hull = nullptr;
     Scratch tmp(c);
     if ((st = tmp.alloc(&d_ang, na)) || (st = tmp.alloc(&d_ent, ent.size())) ||
-        (st = tmp.alloc(&wtab, (size_t)gsz * wtab_angle_floats(c))))
+        (st = tmp.alloc(&hull, (size_t)gsz * hull_angle)))
         return st;
     LMOSEM_CK(c, cudaMemcpyAsync(d_ang, ident.data(), na * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream));
     LMOSEM_CK(c, cudaMemcpyAsync(d_ent, ent.data(), ent.size() * sizeof(int64_t), cudaMemcpyHostToDevice, c->stream));
@@ -1581,18 +1601,20 @@ lmosem_status count_terms(lmosem_ctx* c) {
         const int64_t n_ent = first[gi + 1] - first[gi];
         if (n_ent == 0) continue;
         const int n = std::min(gsz, na - gi * gsz);
-        WTabArgs W = wtab_args(c, wtab, gsz, d_ang, gi * gsz);
+        WTabArgs W = wtab_args(c, nullptr, 0, d_ang, gi * gsz);
+        W.hull = hull;
         if ((st = hull_reset(c, W, n))) return st;
         LMOSEM_PROF_BEGIN(c);
-        k_wtable<<<dim3((c->ld_w + 255) / 256, c->n_scat), 256, 0, c->stream>>>(W, n);
+        k_wtable<false><<<dim3((c->ld_w + 255) / 256, c->n_scat), 256, 0, c->stream>>>(W, n);
         LMOSEM_LAUNCHED(c, LMOSEM_K_WTABLE);
-        TermArgs T{c->d_u_s, c->d_e_s, d_ent + 4 * first[gi], c->d_mpar, W.hull, c->n_scat, W.n_ptiles, c->n_sup,
+        TermArgs T{u, e, d_ent + 4 * first[gi], c->d_mpar, W.hull, c->n_scat, W.n_ptiles, c->n_sup,
                    c->e_sigma > 0.0f ? 1 : 0, c->d_terms};
         LMOSEM_PROF_BEGIN(c);
         k_count_terms<<<dim3((unsigned)n_ent, 32), 256, 0, c->stream>>>(T);
         LMOSEM_LAUNCHED(c, LMOSEM_K_OTHER);
     }
     c->terms_pending = false;
+    drop_kept(c);
     return LMOSEM_OK;
 }
 
@@ -1650,7 +1672,17 @@ lmosem_status exact_rows(lmosem_ctx* c, const std::vector<int64_t>& h_rows, cons
     const bool grid0 = c->use_grid;
     c->use_grid = c->use_grid && as_model;
     st = build_model_rows(c);
-    if (!st && c->terms_pending) st = count_terms(c);  // while these events are in place
+    if (!st && c->terms_pending) {  // these events are not the model's: a copy for the count, should it be asked for
+        c->kept.n_real = c->n_real;
+        c->kept.row0 = c->h_angle_row0;
+        c->kept.cnt = c->h_angle_cnt;
+        if (dev_alloc(c, &c->kept.u, K) || dev_alloc(c, &c->kept.e, K) ||
+            cudaMemcpyAsync(c->kept.u, d_u, K * sizeof(float), cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess ||
+            cudaMemcpyAsync(c->kept.e, d_e, K * sizeof(float), cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess) {
+            drop_kept(c);
+            c->terms_valid = c->terms_pending = false;
+        }
+    }
     c->use_grid = grid0;
     c->use_surrogate = sur0;
     c->fmt = fmt0;
@@ -1851,7 +1883,7 @@ lmosem_status build_binned_rows(lmosem_ctx* c, const int32_t* d_rowmap, int n_eb
             WTabArgs W = wtab_args(c, c->d_wtab, gsz, d_ang, a0);
             if ((st = hull_reset(c, W, na))) return st;  // written by the table kernel, unused here
             LMOSEM_PROF_BEGIN(c);
-            k_wtable<<<dim3((c->ld_w + 255) / 256, c->n_scat), 256, 0, c->stream>>>(W, na);
+            k_wtable<true><<<dim3((c->ld_w + 255) / 256, c->n_scat), 256, 0, c->stream>>>(W, na);
             LMOSEM_LAUNCHED(c, LMOSEM_K_WTABLE);
         }
         for (int a1 = a0; a1 < a0 + na; a1 += msz) {

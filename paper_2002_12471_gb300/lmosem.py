@@ -303,7 +303,8 @@ def lmosem_launch_count(ctx):
 
 
 def lmosem_model_terms(ctx):
-    """Path terms the path-sum kernels formed in the last exact model build."""
+    """Path terms of the last exact model build: counted by the path-sum kernels,
+    or, after a build on the grid, by the first call of this function."""
     n = ctypes.c_int64(0)
     _check(ctx, load().lmosem_model_terms(ctx, ctypes.byref(n)))
     return int(n.value)
