@@ -416,12 +416,14 @@ lmosem_status lmosem_surrogate_check(const lmosem_ctx* ctx, double* h_rel_err, d
  * rows first and the check groups them in energy bins of bin_kev from the
  * window's lower edge; the highest bin whose mean per-row relative L2 error
  * exceeds row_tol marks the cut.  Every model row whose event energy lies
- * below the top of that bin is then built by the exact path sum (bitwise the
- * exact build's row), the others by the network, and the check's error is
- * taken with the former exact.  The exact rows pass through device scratch of
- * at most 8 GiB at a time (ENOMEM from the build when that does not fit).  row_tol = 0: off
- * (the default).  bin_kev = 0 selects 5 keV.  Applies to the builds that
- * follow.  EINVAL: a negative or non-finite argument. */
+ * below the top of that bin is then built exactly, as lmosem_build_model builds
+ * a list of these rows' events alone (path by path, bitwise the row of any such
+ * build; on the grid when they are enough for it), the others by the network,
+ * and the check's error is taken with the former exact.  The exact rows pass
+ * through device scratch of at most 8 GiB at a time (ENOMEM from the build when
+ * that does not fit).  row_tol = 0: off (the default).  bin_kev = 0 selects
+ * 5 keV.  Applies to the builds that follow.  EINVAL: a negative or non-finite
+ * argument. */
 lmosem_status lmosem_set_surrogate_gate(lmosem_ctx* ctx, double row_tol, double bin_kev);
 
 /* Result of the energy gate of the current surrogate-form model:

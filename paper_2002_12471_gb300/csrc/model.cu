@@ -1624,8 +1624,11 @@ lmosem_status count_terms(lmosem_ctx* c) {
 // sum in place of the model's events, and the model's event state is put back
 // after.  The rows of a (realisation, angle) stay contiguous in the sample,
 // and a row's bits do not depend on the other events of its tiles, so every
-// row equals the one the exact build of all events gives (as_model: formed
-// as that build forms them, on the grid or path by path; else path by path).
+// row equals the one the exact build of all events gives path by path.
+// as_model: the rows become the model's; they are then formed on the grid when
+// it pays for a list of K events (for a few rows of a large list it does not:
+// with 10,000 of 250,000 rows below the cut at 128 x 128 the whole surrogate
+// build took 848 ms with their rows on the grid and takes 672 path by path).
 // h_e (K floats, may be NULL) receives the rows' event energies.
 lmosem_status exact_rows(lmosem_ctx* c, const std::vector<int64_t>& h_rows, const int64_t* d_rows, float* d_out,
                          float* h_e, bool as_model) {
@@ -1634,12 +1637,23 @@ lmosem_status exact_rows(lmosem_ctx* c, const std::vector<int64_t>& h_rows, cons
     lmosem_status st;
     int32_t* d_a = nullptr;
     float *d_u = nullptr, *d_e = nullptr;
+    int32_t* d_out_n = nullptr;
     Scratch tmp(c);
-    if ((st = tmp.alloc(&d_a, K)) || (st = tmp.alloc(&d_u, K)) || (st = tmp.alloc(&d_e, K))) return st;
+    if ((st = tmp.alloc(&d_a, K)) || (st = tmp.alloc(&d_u, K)) || (st = tmp.alloc(&d_e, K)) ||
+        (st = tmp.alloc(&d_out_n, 1)))
+        return st;
     LMOSEM_PROF_BEGIN(c);
     k_judge_gather<<<(unsigned)((K + 255) / 256), 256, 0, c->stream>>>(c->d_a_s, c->d_u_s, c->d_e_s, d_rows, K,
                                                                         d_a, d_u, d_e);
     LMOSEM_LAUNCHED(c, LMOSEM_K_OTHER);
+    bool grid = false;
+    int32_t n_outside = 0;
+    if (as_model && c->use_grid && (st = grid_plan(c, K, &grid))) return st;
+    if (grid) {
+        LMOSEM_CK(c, cudaMemsetAsync(d_out_n, 0, sizeof(int32_t), c->stream));
+        if ((st = grid_count_outside(c, d_a, d_u, d_e, K, d_out_n))) return st;
+        LMOSEM_CK(c, cudaMemcpyAsync(&n_outside, d_out_n, sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
+    }
     std::vector<int32_t> h_a(K);
     LMOSEM_CK(c, cudaMemcpyAsync(h_a.data(), d_a, K * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
     if (h_e) LMOSEM_CK(c, cudaMemcpyAsync(h_e, d_e, K * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
@@ -1670,7 +1684,9 @@ lmosem_status exact_rows(lmosem_ctx* c, const std::vector<int64_t>& h_rows, cons
     c->fmt = LMOSEM_MODEL_FP32;
     c->use_surrogate = false;
     const bool grid0 = c->use_grid;
-    c->use_grid = c->use_grid && as_model;
+    const int64_t direct0 = c->grid_max_direct;
+    c->use_grid = grid && n_outside <= c->grid.max_direct;
+    c->grid_max_direct = c->grid.max_direct - n_outside;
     st = build_model_rows(c);
     if (!st && c->terms_pending) {  // these events are not the model's: a copy for the count, should it be asked for
         c->kept.n_real = c->n_real;
@@ -1684,6 +1700,7 @@ lmosem_status exact_rows(lmosem_ctx* c, const std::vector<int64_t>& h_rows, cons
         }
     }
     c->use_grid = grid0;
+    c->grid_max_direct = direct0;
     c->use_surrogate = sur0;
     c->fmt = fmt0;
     c->d_model = m0;
