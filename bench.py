@@ -163,12 +163,17 @@ def strip_terms(ph, g, ev, k_sigma=6.0):
     return total * n_nz, n_nz
 
 
-def grid_sum_flops(ph, g, k_sigma=6.0):
+def grid_sum_flops(ph, g):
     """Operations of the scatter sum in its grid form, without padding: per
     angle, support pixel and energy node one multiply-add for every position
-    node within k_sigma sigma_u(m) of each scatter pixel m, as three products
-    of 16-bit parts.  Nodes 0.415 of the narrowest sigma_u apart, and 1/4
-    apart in 2 sqrt(E / kappa) (sigma_E^2 = kappa E)."""
+    node that the response of a scatter pixel reaches, as three products of
+    16-bit parts.  The grid as the library plans it at the default cuts:
+    responses cut at 6 sigma_u(m) and at 5.5 of the widest; the position step
+    from a window of 96 nodes, which holds the widest response and a subgroup
+    of scatter pixels; energy nodes 1/4 apart in 2 sqrt(E / kappa) (sigma_E^2 =
+    kappa E) over the part of the window that events reach, 7 of them beyond
+    its cells for the stencil."""
+    from paper_2002_12471_gb300 import synthetic as S
     mu = ph.mu.reshape(-1)
     ny, nx = ph.mu.shape
     scat = np.nonzero(mu > 0)[0]
@@ -176,15 +181,44 @@ def grid_sum_flops(ph, g, k_sigma=6.0):
     y = (scat // nx + 0.5 - 0.5 * ny) * ph.pixel_mm
     fw2s = 1.0 / 2.3548200450309493
     rmax = float(np.sqrt((x * x + y * y).max()))
-    s_min = (g["coll_fwhm0_mm"] + g["coll_fwhm_slope"] * (g["radius_mm"] - rmax)) * fw2s
+    s_min, s_max = ((g["coll_fwhm0_mm"] + g["coll_fwhm_slope"] * (g["radius_mm"] + r)) * fw2s for r in (-rmax, rmax))
+    cut = 5.5 * s_max
+    span = min(87 * 0.415 * s_min - 2.0 * cut, 1.25 * 64 * 2.0 * rmax / len(scat))
+    step = max((2.0 * cut + span) / 87, 0.30 * s_min)
     kappa = (g["fwhm_frac_e0"] * fw2s) ** 2 * g["e0_kev"]
-    nodes_e = (2.0 * np.sqrt(g["e_hi_kev"] / kappa) - 2.0 * np.sqrt(g["e_lo_kev"] / kappa)) / 0.25
+    e_back = g["e0_kev"] / (1.0 + 2.0 * g["e0_kev"] / S.MEC2_KEV)
+    e_min = max(g["e_lo_kev"], e_back - 1.5 * np.sqrt(kappa * e_back))
+    e_max = min(g["e_hi_kev"], g["e0_kev"] + 3.0 * np.sqrt(kappa * g["e0_kev"]))
+    nodes_e = int((2.0 * np.sqrt(e_max / kappa) - 2.0 * np.sqrt(e_min / kappa)) / 0.25) + 1 + 7
     total = 0.0
     for a in range(g["n_angles"]):
         th = g["angle0_rad"] + 2 * np.pi * a / g["n_angles"]
         sig = (g["coll_fwhm0_mm"] + g["coll_fwhm_slope"] * (g["radius_mm"] - (x * np.cos(th) + y * np.sin(th)))) * fw2s
-        total += float((2.0 * k_sigma * sig / (0.415 * s_min)).sum())
+        total += float((2.0 * np.minimum(6.0 * sig, cut) / step).sum())
     return 3 * 2 * total * nodes_e * len(scat)
+
+
+def build_roofline(on_grid, ph, g, events, ms, terms, terms_exact, ex2_peak, ex2_basis, pk, pk_kind):
+    """Roofline of the row build of one step (ms of its path-sum class kernels):
+    of the form that the library says it took."""
+    rate = terms / (ms * 1e-3) / 1e9          # Gterm/s
+    if not on_grid:
+        return {"bound": "alu", "kernel": "k_pathsum", "achieved": rate, "peak": ex2_peak,
+                "unit": "Gterm/s", "frac": rate / ex2_peak,
+                "traffic": read_traffic("k_pathsum", "%s_%gM" % (WORKLOAD, events / 1e6)),
+                "peak_basis": ex2_basis,
+                "units": "path terms the position and energy cuts keep (counted by the kernels)",
+                "exact_sum_terms_frac": rate * (terms_exact / terms) / ex2_peak,
+                "exact_sum_terms_note": "the exact sum's terms (position strip only) per second of "
+                                        "the same kernel time, over the same peak: the rate at "
+                                        "which the cut delivers the exact sum's result"}
+    tf = grid_sum_flops(ph, g) / (ms * 1e-3) / 1e12
+    return {"bound": "tensor", "kernel": "k_grid_sum + k_grid_rows", "achieved": tf,
+            "peak": pk["bf16_tflops"], "unit": "TFLOP/s", "frac": tf / pk["bf16_tflops"], "traffic": None,
+            "peak_kind": pk_kind + " burst BF16",
+            "units": "three 16-bit products per (grid node, scatter pixel, support pixel) within the "
+                     "position cut, over the time of the products and of the interpolation at the events",
+            "equivalent_gterm_per_s": rate}
 
 
 # ------------------------------------------------------------------ clocks
@@ -397,7 +431,7 @@ def run_ours(args, rank, world, local_rank):
 
     budget = args.table_budget_mb << 20
 
-    kept_terms = {}
+    kept_terms, on_grid = {}, {}
 
     def step(fmt, a, u, e, profile=0, count=False):
         ctx = L.lmosem_create(ph.mu, ph.pixel_mm, g, stream=stream, e_sigma=args.e_sigma, profile=profile,
@@ -408,6 +442,7 @@ def run_ours(args, rank, world, local_rank):
             L.lmosem_build_model(ctx, a, u, e, ns, fmt)
             if count:   # untimed steps only: the count synchronises the stream
                 kept_terms[fmt] = L.lmosem_model_terms(ctx)
+                on_grid[fmt] = L.lmosem_model_on_grid(ctx)
             f = torch.empty(nsup, dtype=torch.float32, device=dev)
             ll = torch.empty(1, dtype=torch.float64, device=dev)
             L.lmosem_init_image(ctx, T, f)
@@ -580,30 +615,10 @@ def run_ours(args, rank, world, local_rank):
     agg, pass_ms, pass_n, pass_gbs, ms_step = summary(chosen)
     tot_kernel_ms = sum(v[0] for v in agg.values())
     ps_ms, ps_n = agg["pathsum"]
-    ps_launch_ms = ps_ms / max(1, ps_n)
-    terms_per_launch = terms / max(1, ps_n / args.steps)
-    achieved = terms_per_launch / (ps_launch_ms * 1e-3) / 1e9          # Gterm/s
     peak = MUFU_EX2_PER_CLK_SM * sms * sm_max * 1e6 / 1e9             # Gterm/s (1 ex2 / term)
-    if achieved < peak:
-        roofline = {"bound": "alu", "kernel": "k_pathsum", "achieved": achieved, "peak": peak,
-                    "unit": "Gterm/s", "frac": achieved / peak,
-                    "traffic": read_traffic("k_pathsum", "%s_%gM" % (WORKLOAD, J / 1e6)),
-                    "peak_basis": "%d MUFU ex2 per clock per SM x %d SMs x %.0f MHz; one ex2 and "
-                                  "three FP32 FMAs per path term" % (MUFU_EX2_PER_CLK_SM, sms, sm_max),
-                    "units": "path terms the position and energy cuts keep (counted by the kernels)",
-                    "exact_sum_terms_frac": achieved * (terms_exact / terms) / peak,
-                    "exact_sum_terms_note": "the exact sum's terms (position strip only) per second of "
-                                            "the same kernel time, over the same peak: the rate at "
-                                            "which the cut delivers the exact sum's result"}
-    else:  # more terms than the exponential unit could form: the sum was formed on the grid
-        flops = grid_sum_flops(ph, g)
-        tf = flops / (ps_ms / args.steps * 1e-3) / 1e12
-        roofline = {"bound": "tensor", "kernel": "k_grid_sum + k_grid_rows", "achieved": tf,
-                    "peak": pk["bf16_tflops"], "unit": "TFLOP/s", "frac": tf / pk["bf16_tflops"], "traffic": None,
-                    "peak_kind": pk_kind + " burst BF16",
-                    "units": "three 16-bit products per (grid node, scatter pixel, support pixel) within the "
-                             "position cut, over the time of the products and of the interpolation at the events",
-                    "equivalent_gterm_per_s": achieved}
+    roofline = build_roofline(on_grid[chosen], ph, g, J, ps_ms / args.steps, terms, terms_exact, peak,
+                              "%d MUFU ex2 per clock per SM x %d SMs x %.0f MHz; one ex2 and three FP32 FMAs per "
+                              "path term" % (MUFU_EX2_PER_CLK_SM, sms, sm_max), pk, pk_kind)
     value = aggregate_rate(evals, world, ms_step)
     e2e_ms = statistics.mean(e2e_times)
     R = runs[chosen]
@@ -630,7 +645,7 @@ def run_ours(args, rank, world, local_rank):
                               "model_bytes": R["model_bytes"]},
         "breakdown_ms_per_step": {k: v[0] / args.steps for k, v in agg.items() if v[1]},
         "kernel_share": {k: v[0] / tot_kernel_ms for k, v in agg.items() if v[1]},
-        "model_build_evals_per_s": evals / (ps_launch_ms * ps_n / args.steps * 1e-3),
+        "model_build_evals_per_s": evals / (ps_ms / args.steps * 1e-3),
         "path_terms_per_step": terms,
         "path_terms_exact_sum_per_step": terms_exact,
         "energy_cut_kept_frac": terms / terms_exact,

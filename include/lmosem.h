@@ -507,6 +507,11 @@ int64_t lmosem_launch_count(const lmosem_ctx* ctx);
  * rows have been built on this context. */
 lmosem_status lmosem_model_terms(lmosem_ctx* ctx, int64_t* h_terms);
 
+/* Which form the last row build took (the rows that lmosem_model_terms counts):
+ * *h_on_grid = 1 when it formed the scatter sum on the grid, 0 when path by
+ * path.  EINVAL: no exact rows have been built on this context. */
+lmosem_status lmosem_model_on_grid(lmosem_ctx* ctx, int32_t* h_on_grid);
+
 /* Change the clock-cycle budget of the bounded device waits (see
  * lmosem_options.wait_budget_cycles; 0 restores 2e9) for the calls that
  * follow, e.g. to let a test build the model and then make one pass time

@@ -309,6 +309,13 @@ lmosem_status lmosem_model_terms(lmosem_ctx* c, int64_t* h_terms) {
     return LMOSEM_OK;
 }
 
+lmosem_status lmosem_model_on_grid(lmosem_ctx* c, int32_t* h_on_grid) {
+    if (!c || !h_on_grid) return LMOSEM_EINVAL;
+    if (!c->terms_valid) return fail(c, LMOSEM_EINVAL, "no exact model build to ask about");
+    *h_on_grid = c->rows_on_grid ? 1 : 0;
+    return LMOSEM_OK;
+}
+
 int64_t lmosem_model_bytes(const lmosem_ctx* ctx) {
     if (!ctx || ctx->fmt < 0) return 0;
     int64_t elem = ctx->fmt == LMOSEM_MODEL_FP32 ? 4 : 2;

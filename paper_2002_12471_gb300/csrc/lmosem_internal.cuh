@@ -143,6 +143,7 @@ struct lmosem_ctx {
     lmosem::GridPlan grid;
     bool use_grid = false;        // the model's exact rows come from the grid
     int64_t grid_max_direct = 0;  // steep rows of it that may be summed directly
+    bool rows_on_grid = false;    // the last exact rows were formed on the grid
     bool grid_expected = false;   // the next build's will: the sensitivity leaves the scatter planes out
     int* d_status = nullptr;      // [0] = 1 after a bounded device wait ran out
     long long wait_budget = 2000000000LL;  // clock cycles per bounded wait

@@ -1286,12 +1286,12 @@ lmosem_status build_model_rows(lmosem_ctx* c) {
         st = build_model_rows_grid(c, slot_angle, c->grid_max_direct, &done);
         if (st != LMOSEM_ENOMEM && (st || done)) {
             drop_kept(c);
-            c->terms_valid = c->terms_pending = st == LMOSEM_OK;
+            c->terms_valid = c->terms_pending = c->rows_on_grid = st == LMOSEM_OK;
             return st;
         }
         c->use_grid = false;  // its buffers do not fit beside the model, or too many rows are steep: path by path
     }
-    c->terms_pending = false;
+    c->terms_pending = c->rows_on_grid = false;
     drop_kept(c);
 
     // angle groups bounded by the scatter-table budget (three FP32 planes);

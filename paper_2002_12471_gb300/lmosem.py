@@ -96,6 +96,7 @@ SIGNATURES = {
     "lmosem_model_bytes": (_i64, [_vp]),
     "lmosem_launch_count": (_i64, [_vp]),
     "lmosem_model_terms": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_int64)]),
+    "lmosem_model_on_grid": (ctypes.c_int, [_vp, ctypes.POINTER(_i32)]),
     "lmosem_set_wait_budget": (ctypes.c_int, [_vp, _i64]),
     "lmosem_subset_totals": (ctypes.c_int, [_vp, _dbl, _vp, _vp]),
     "lmosem_profile_read": (ctypes.c_int, [_vp, _vp, _vp]),
@@ -308,6 +309,13 @@ def lmosem_model_terms(ctx):
     n = ctypes.c_int64(0)
     _check(ctx, load().lmosem_model_terms(ctx, ctypes.byref(n)))
     return int(n.value)
+
+
+def lmosem_model_on_grid(ctx):
+    """Whether the last exact model build formed the scatter sum on the grid."""
+    n = _i32(0)
+    _check(ctx, load().lmosem_model_on_grid(ctx, ctypes.byref(n)))
+    return bool(n.value)
 
 
 def lmosem_set_wait_budget(ctx, cycles):
