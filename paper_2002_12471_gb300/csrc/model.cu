@@ -168,9 +168,13 @@ struct WSensArgs {
 
 // Blocks of kFuseX columns x kFuseY shares: share y takes the 32-pixel pieces
 // y, y + kFuseY, ... of the scatter pixels (the FP32 sums of a piece go
-// through shared memory and are added in order), so that a small problem
-// fills more than a few warps (16 x 16: 110 us with one share).
-constexpr int kFuseX = 64, kFuseY = 8;
+// through shared memory and are added in order, kFusePieces at a time), so that
+// a small problem fills more than a few warps (16 x 16: 110 us with one share).
+// MANY: more than kFusePieces pieces, in rounds (the others without the loop,
+// which changes the code of the pieces: 63 instead of 40 to 52 registers, and 20
+// to 90 us less at 50 x 50 with 90 angles).
+constexpr int kFuseX = 64, kFuseY = 8, kFusePieces = 128;
+template <bool MANY>
 __global__ void __launch_bounds__(kFuseX * kFuseY) k_wtable_sens(WSensArgs S) {
     extern __shared__ float pieces[];  // [piece][kFuseX]
     const WTabArgs& A = S.w;
@@ -187,41 +191,51 @@ __global__ void __launch_bounds__(kFuseX * kFuseY) k_wtable_sens(WSensArgs S) {
     const float* le = A.l_edge + (size_t)a * A.npix;
     const float* du = S.du_m + (size_t)a * A.n_scat;
     const int n_pieces = (A.n_scat + 31) / 32;
-    for (int p = threadIdx.y; p < n_pieces; p += kFuseY) {
-        float part = 0.0f;
-        for (int k = 32 * p; k < min(A.n_scat, 32 * p + 32); ++k) {
-            const float4 gm = __ldg(A.scat_geo + k);
-            const int pm = __float_as_int(gm.w);
-            float s = 0.0f, b = 0.0f, nlw = INFINITY;
-            uint2 hb = make_uint2(0xffffffffu, 0xffffffffu);
-            float cpsi, rinv;
-            if (real && path_geometry_xy(xn, yn, gm.x, gm.y, pn == pm, trig, &cpsi, &rinv)) {
-                float P, kt;
-                compton(cpsi, A.eps0, A.inv_kbar, &P, &kt);
-                const float2 cr = compton_lookup(A.compton, cpsi);  // (mu ratio, window mass)
-                const float att = fmaf(cr.x, __ldg(le + pm), lp[(size_t)k * A.n_sup]);
-                const float mu = gm.z;
-                const float e1 = A.e0 * P;
-                const float ri = rsqrtf(e1);
-                nlw = fmaf(att, kLog2e, -__log2f(A.w_const * mu * kt * rinv * ri));
-                s = A.cE * ri;
-                b = -e1 * s;
-                hb = hull_bits(e1, ri, A.hK);
-                const float w = S.w_const_sens * mu * kt * rinv * __expf(-att);
-                part = fmaf(w, __ldg(du + k) * cr.y, part);
+    double acc = 0.0;
+    int p0 = 0;
+    do {  // once unless MANY
+        const int p1 = MANY ? min(n_pieces, p0 + kFusePieces) : n_pieces;
+        for (int p = (MANY ? p0 : 0) + threadIdx.y; p < p1; p += kFuseY) {
+            float part = 0.0f;
+            for (int k = 32 * p; k < min(A.n_scat, 32 * p + 32); ++k) {
+                const float4 gm = __ldg(A.scat_geo + k);
+                const int pm = __float_as_int(gm.w);
+                float s = 0.0f, b = 0.0f, nlw = INFINITY;
+                uint2 hb = make_uint2(0xffffffffu, 0xffffffffu);
+                float cpsi, rinv;
+                if (real && path_geometry_xy(xn, yn, gm.x, gm.y, pn == pm, trig, &cpsi, &rinv)) {
+                    float P, kt;
+                    compton(cpsi, A.eps0, A.inv_kbar, &P, &kt);
+                    const float2 cr = compton_lookup(A.compton, cpsi);  // (mu ratio, window mass)
+                    const float att = fmaf(cr.x, __ldg(le + pm), lp[(size_t)k * A.n_sup]);
+                    const float mu = gm.z;
+                    const float e1 = A.e0 * P;
+                    const float ri = rsqrtf(e1);
+                    nlw = fmaf(att, kLog2e, -__log2f(A.w_const * mu * kt * rinv * ri));
+                    s = A.cE * ri;
+                    b = -e1 * s;
+                    hb = hull_bits(e1, ri, A.hK);
+                    const float w = S.w_const_sens * mu * kt * rinv * __expf(-att);
+                    part = fmaf(w, __ldg(du + k) * cr.y, part);
+                }
+                base[(size_t)k * A.ld_w] = s;
+                base[plane + (size_t)k * A.ld_w] = b;
+                base[2 * plane + (size_t)k * A.ld_w] = nlw;
+                hull_fold(hull + k, hb);
             }
-            base[(size_t)k * A.ld_w] = s;
-            base[plane + (size_t)k * A.ld_w] = b;
-            base[2 * plane + (size_t)k * A.ld_w] = nlw;
-            hull_fold(hull + k, hb);
+            pieces[(MANY ? p - p0 : p) * kFuseX + threadIdx.x] = part;
         }
-        pieces[p * kFuseX + threadIdx.x] = part;
-    }
-    __syncthreads();
-    if (threadIdx.y != 0 || !real) return;
-    double acc = (double)(expf(-A.l_edge[(size_t)a * A.npix + pn]) * S.ppar[(size_t)a * A.ld_w + n].w * S.de0);
-    for (int p = 0; p < n_pieces; ++p) acc += (double)pieces[p * kFuseX + threadIdx.x];
-    S.sens_angle[(size_t)a * A.n_sup + n] = acc;
+        __syncthreads();
+        if (!MANY && (threadIdx.y != 0 || !real)) return;
+        if (!MANY || (threadIdx.y == 0 && real)) {
+            if (p0 == 0)
+                acc = (double)(expf(-A.l_edge[(size_t)a * A.npix + pn]) * S.ppar[(size_t)a * A.ld_w + n].w * S.de0);
+            for (int p = 0; p < p1 - p0; ++p) acc += (double)pieces[p * kFuseX + threadIdx.x];
+        }
+        p0 = p1;
+        if (MANY) __syncthreads();  // before the pieces are overwritten
+    } while (MANY && p0 < n_pieces);
+    if (threadIdx.y == 0 && real) S.sens_angle[(size_t)a * A.n_sup + n] = acc;
 }
 
 struct PathSumArgs {
@@ -1225,7 +1239,7 @@ lmosem_status hull_reset(lmosem_ctx* c, const WTabArgs& W, int n) {
 // whole reconstruction 4.83 ms, 5.07 with sensitivity and planes apart).
 bool wtab_all_fits(const lmosem_ctx* c) {
     const int64_t bytes = (int64_t)c->n_angles * wtab_angle_floats(c) * (int64_t)sizeof(float);
-    return !c->grid_expected && bytes <= c->table_budget && c->n_scat <= 32 * 128;
+    return !c->grid_expected && bytes <= c->table_budget;
 }
 
 lmosem_status wtab_all_with_sens(lmosem_ctx* c, double* sens_angle, float w_const_sens, float de0) {
@@ -1240,8 +1254,12 @@ lmosem_status wtab_all_with_sens(lmosem_ctx* c, double* sens_angle, float w_cons
     S.de0 = de0;
     S.sens_angle = sens_angle;
     LMOSEM_PROF_BEGIN(c);
-    const size_t smem = sizeof(float) * kFuseX * ((c->n_scat + 31) / 32);
-    k_wtable_sens<<<dim3(c->ld_w / kFuseX, c->n_angles), dim3(kFuseX, kFuseY), smem, c->stream>>>(S);
+    // (no more than needed: with the full 32 KB, L1 is short of the pair integrals and 50 x 50 with 90 angles takes
+    // 40 us more)
+    const int n_pieces = (c->n_scat + 31) / 32;
+    const size_t smem = sizeof(float) * kFuseX * std::min(kFusePieces, n_pieces);
+    auto kern = n_pieces > kFusePieces ? k_wtable_sens<true> : k_wtable_sens<false>;
+    kern<<<dim3(c->ld_w / kFuseX, c->n_angles), dim3(kFuseX, kFuseY), smem, c->stream>>>(S);
     LMOSEM_LAUNCHED(c, LMOSEM_K_SENS);
     return LMOSEM_OK;
 }
