@@ -239,6 +239,22 @@ void prof_end(lmosem_ctx* c, int cls);
             return ::lmosem::cuda_fail(ctx, e_, "launch at " __FILE__ ":" LMOSEM_STR(__LINE__)); \
     } while (0)
 
+// Lets `kern` be launched with `bytes` of dynamic shared memory.  The limit
+// belongs to the function and not to the context, so it is only ever raised, to
+// the most that the function can take: a limit set to each context's own size
+// could be lowered by another host thread between the call and the launch.
+template <typename F>
+lmosem_status opt_in_smem(lmosem_ctx* c, F* kern, size_t bytes) {
+    cudaFuncAttributes fa;
+    LMOSEM_CK(c, cudaFuncGetAttributes(&fa, kern));
+    if (bytes <= (size_t)fa.maxDynamicSharedSizeBytes) return LMOSEM_OK;
+    int dev = 0, most = 0;
+    LMOSEM_CK(c, cudaGetDevice(&dev));
+    LMOSEM_CK(c, cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    LMOSEM_CK(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes));
+    return LMOSEM_OK;
+}
+
 // Device memory of a context is stream-ordered on the context's stream
 // (cudaMallocAsync / cudaFreeAsync from the device's default pool, which keeps
 // up to kPoolKeepBytes cached between calls): a buffer may be freed right
