@@ -251,8 +251,8 @@ lmosem_status build_model_common(lmosem_ctx* c, const int32_t* d_angle, const fl
         return st;
     }
     // the rows outside the grid's region are among those summed directly
-    c->use_grid = grid && n_outside <= c->grid.max_direct;
-    c->grid_max_direct = c->grid.max_direct - n_outside;
+    c->grid_ratio = c->grid.ratio + kDirectCost * n_outside / n_events;
+    c->use_grid = grid && c->grid_ratio < kGridGain;
     if ((st = sur ? build_checked_surrogate(c) : build_model_rows(c))) {
         free_model(c);
         return st;

@@ -841,10 +841,12 @@ struct RowArgs {
 
 // Rows of 64 events (in block order) x 128 support pixels: the 13 x 9 grid
 // values around a block of 2 x 2 cells are loaded once for all of its events.
-// Instructions bound the kernel (about 250 issue slots per event and warp when
-// the stencil of an odd cell was copied to even registers): blocks of 2 x 2
+// The values take 166 registers, so 12 warps per SM; what bounds the kernel is
+// each warp's own chain: 47% of the issue slots are used, 2.2 cycles per
+// instruction go to fixed latencies and 0.9 to loads.  Fewer instructions per
+// event shorten it: blocks of 2 x 2
 // cells hold about twice the events of a cell for 1.2 times the values (per 33k
-// events x 5,884 pixels 1.97 -> 1.78 ms), and an odd cell shifts its 12 weights
+// events at 128 x 128 1.97 -> 1.78 ms), and an odd cell shifts its 12 weights
 // instead of 96 values (model build of 250k events at 128 x 128 50.0 -> 48.7 ms,
 // of 450k at 64 x 64 9.20 -> 8.57), and the sum over the energy nodes comes
 // first, packed throughout (48.7 -> 48.4, 8.57 -> 8.40).  Slower: larger blocks (53.6 to 54.9 ms; 174
@@ -1161,9 +1163,9 @@ CellArgs cell_args(const lmosem_ctx* c, const int32_t* a, const float* u, const 
 //    being kept by the energy cut.
 // They meet near 500 events per angle at 128 x 128 (6,000 pixels) and near
 // 1,000 at 64 x 64 (1,540); the grid has to win by a tenth, with every row that
-// is summed directly (k_grid_direct) counted as 30 of the path sum's: at most
-// max_direct of them.  (Measured: 2.5 path-sum rows each for 1,000 at the edge of
-// the object at 64 x 64, more inside it, and the latency of one per group, 40 us.)
+// is summed directly (k_grid_direct) counted as kDirectCost of the path sum's.
+// (Measured: 2.5 path-sum rows each for 1,000 at the edge of the object at 64 x
+// 64, more inside it, and the latency of one per group, 40 us.)
 lmosem_status grid_plan(lmosem_ctx* c, int64_t n, bool* use) {
     *use = false;
     if (n < (int64_t)64 * c->n_angles || c->n_scat < 2 * kSub || c->n_scat > 16384) return LMOSEM_OK;
@@ -1228,8 +1230,8 @@ lmosem_status grid_plan(lmosem_ctx* c, int64_t n, bool* use) {
     const double t_grid = c->n_angles * ((c->n_sup + kNTile - 1) / kNTile * (G.ne / kEGroup) * (2300.0 * G.n_sub + 9000.0) / per_s +
                                          tiles * G.n_sub * 25e-9) + n * tiles * 400.0 / per_s + 60e-6;
     const double t_path = n * (0.8 * G.strip * c->n_scat * c->n_sup) / 5.5e12;
-    if (!(t_grid < 0.9 * t_path)) return LMOSEM_OK;
-    G.max_direct = (int64_t)((0.9 - t_grid / t_path) * n / 30.0);
+    G.ratio = t_grid / t_path;
+    if (!(G.ratio < kGridGain)) return LMOSEM_OK;
     *use = true;
     if (G.state == 3) return LMOSEM_OK;
     const double kappa = kappa_of(c);
@@ -1293,10 +1295,12 @@ lmosem_status grid_count_outside(lmosem_ctx* c, const int32_t* a, const float* u
 }
 
 // Rows of every sorted event (scaled forms: staged as FP32 per group and
-// rounded), angle group by angle group within the table budget.  *done = false:
-// too many rows are steep (more than max_direct, or so many in the first group), and the path sum has to form them all.
-lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& slot_angle, int64_t max_direct,
-                                    bool* done) {
+// rounded), angle group by angle group within the table budget.  ratio: the
+// list's cost here over the path sum's, before any row is known to be steep.
+// *done = false: so many rows are steep that the path sum forms the whole list
+// faster than what is left to do here (looked at once, after the first group),
+// or than their direct sums (at the end).
+lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& slot_angle, double ratio, bool* done) {
     const GridPlan& G = c->grid;
     *done = false;
     lmosem_status st;
@@ -1348,7 +1352,7 @@ lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& s
     float4* planes = nullptr;
     float* T = nullptr;
     unsigned char* ublob = nullptr;
-    const int max_list = (int)std::max<int64_t>(0, std::min<int64_t>(max_direct, J));
+    const int max_list = (int)(J / kDirectCost);
     const int n_groups = (ns + gsz - 1) / gsz;
     int32_t *list = nullptr, *n_list = nullptr;  // n_list[0]: rows found; [1 + gi]: before group gi
     float *pmax = nullptr, *top = nullptr;
@@ -1551,7 +1555,8 @@ lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& s
             looked = true;
             LMOSEM_CK(c, cudaMemcpyAsync(&found, n_list, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
             LMOSEM_CK(c, cudaStreamSynchronize(c->stream));
-            if (found > 32 && (double)found * J > (double)max_list * rows_done) break;
+            const double f = (double)rows_done / (double)J;
+            if (found > 32 && (1.0 - f) * ratio + kDirectCost * found / (f * J) > 1.0) break;
         }
     }
     dev_free(c, &c->d_stage);

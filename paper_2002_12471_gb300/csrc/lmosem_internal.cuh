@@ -47,7 +47,7 @@ struct GridPlan {
     double edge = 0, e_min = 0, e_max = 0;  // events beyond are summed directly
     int max_sub = 0, n_sub = 0;  // subgroups per angle at most, and about
     double strip = 0;            // share of the scatter pixels within an event's position cut
-    int64_t max_direct = 0;      // rows of the last planned list that may be summed directly
+    double ratio = 0;            // cost of the last planned list on the grid / by the path sum
     float log_g = 0, log_u = 0;  // log2 of the operands' scales
     int32_t* d_slot_m = nullptr; // [a][subgroup][64]: scatter pixel or -1
     int32_t* d_i0 = nullptr;     // [a][subgroup]: first node
@@ -142,7 +142,7 @@ struct lmosem_ctx {
     lmosem::TermEvents kept;      // (u set) the pending count's events, no longer the model's
     lmosem::GridPlan grid;
     bool use_grid = false;        // the model's exact rows come from the grid
-    int64_t grid_max_direct = 0;  // steep rows of it that may be summed directly
+    double grid_ratio = 0;        // its cost there, the rows outside the grid's region included / the path sum's
     bool rows_on_grid = false;    // the last exact rows were formed on the grid
     bool grid_expected = false;   // the next build's will: the sensitivity leaves the scatter planes out
     int* d_status = nullptr;      // [0] = 1 after a bounded device wait ran out
@@ -363,12 +363,13 @@ lmosem_status sort_events(lmosem_ctx* c, const int32_t* d_angle, const float* d_
 int64_t scan_blocks(int64_t n);
 lmosem_status exclusive_scan(lmosem_ctx* c, int32_t* x, int64_t n, int32_t* tot);
 // grid.cu
+constexpr double kDirectCost = 30.0;  // a directly summed row, in rows of the path sum (see grid_plan)
+constexpr double kGridGain = 0.9;     // the grid is taken below this share of the path sum's time
 lmosem_status grid_plan(lmosem_ctx* c, int64_t n_events, bool* use);
 void grid_free(lmosem_ctx* c);
 lmosem_status grid_count_outside(lmosem_ctx* c, const int32_t* a, const float* u, const float* e, int64_t n,
                                  int32_t* d_n);
-lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& slot_angle, int64_t max_direct,
-                                    bool* done);
+lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& slot_angle, double ratio, bool* done);
 // model.cu: staged FP32 rows (d_stage) to the scaled rows row0 ..; path terms of the pending count's events
 lmosem_status quantize_rows(lmosem_ctx* c, int64_t rows, int64_t row0);
 lmosem_status count_terms(lmosem_ctx* c);

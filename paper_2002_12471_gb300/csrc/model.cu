@@ -1301,7 +1301,7 @@ lmosem_status build_model_rows(lmosem_ctx* c) {
     if (c->use_grid && !c->scatter_only) {
         dev_free(c, &c->d_wtab_all);  // the grid has tables of its own
         bool done = false;
-        st = build_model_rows_grid(c, slot_angle, c->grid_max_direct, &done);
+        st = build_model_rows_grid(c, slot_angle, c->grid_ratio, &done);
         if (st != LMOSEM_ENOMEM && (st || done)) {
             drop_kept(c);
             c->terms_valid = c->terms_pending = c->rows_on_grid = st == LMOSEM_OK;
@@ -1701,9 +1701,9 @@ lmosem_status exact_rows(lmosem_ctx* c, const std::vector<int64_t>& h_rows, cons
     c->fmt = LMOSEM_MODEL_FP32;
     c->use_surrogate = false;
     const bool grid0 = c->use_grid;
-    const int64_t direct0 = c->grid_max_direct;
-    c->use_grid = grid && n_outside <= c->grid.max_direct;
-    c->grid_max_direct = c->grid.max_direct - n_outside;
+    const double ratio0 = c->grid_ratio;
+    c->grid_ratio = c->grid.ratio + kDirectCost * n_outside / K;
+    c->use_grid = grid && c->grid_ratio < kGridGain;
     st = build_model_rows(c);
     if (!st && c->terms_pending) {  // these events are not the model's: a copy for the count, should it be asked for
         c->kept.n_real = c->n_real;
@@ -1717,7 +1717,7 @@ lmosem_status exact_rows(lmosem_ctx* c, const std::vector<int64_t>& h_rows, cons
         }
     }
     c->use_grid = grid0;
-    c->grid_max_direct = direct0;
+    c->grid_ratio = ratio0;
     c->use_surrogate = sur0;
     c->fmt = fmt0;
     c->d_model = m0;
