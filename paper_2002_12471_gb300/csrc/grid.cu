@@ -1260,7 +1260,7 @@ lmosem_status grid_plan(lmosem_ctx* c, int64_t n, bool* use) {
     k_grid_rank<<<dim3((c->n_scat + 255) / 256, c->n_angles), 256, 0, c->stream>>>(c->d_mpar, c->n_scat, order);
     LMOSEM_LAUNCHED(c, LMOSEM_K_TABLES);
     const size_t smem = sizeof(float) * ((size_t)c->n_scat + G.max_sub + 1);
-    if ((st = opt_in_smem(c, k_grid_groups, smem))) return st;
+    if ((st = opt_in_smem(c, k_grid_groups))) return st;
     LMOSEM_PROF_BEGIN(c);
     k_grid_groups<<<c->n_angles, 256, smem, c->stream>>>(
         c->d_mpar, order, c->n_scat, G.max_sub, (float)G.span, (float)G.cut,
@@ -1383,7 +1383,7 @@ lmosem_status build_model_rows_grid(lmosem_ctx* c, const std::vector<int32_t>& s
     if (scaled && (st = dev_alloc(c, &c->d_stage, (size_t)std::max<int64_t>(
                                                        1, *std::max_element(g_rows.begin(), g_rows.end())) * ld)))
         return st;
-    if ((st = opt_in_smem(c, k_grid_sum, kSmBytes))) return st;
+    if ((st = opt_in_smem(c, k_grid_sum))) return st;
     const float cE2 = (float)(1.4426950408889634 / (2.0 * kappa));
     int64_t rows_done = 0;
     bool looked = false;

@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -162,6 +163,7 @@ struct lmosem_ctx {
     int surrogate_kernel = 0;                 // inference: 0 auto (fused tcgen05), 1 product chain, 2 fused
     int prefetch_groups = 0;                  // register pass: groups prefetched into L2 ahead (-1 none, 0 auto)
     bool gemm_attrs = false;                  // shared-memory opt-in of the training products is set
+    std::vector<const void*> smem_raised;     // kernels whose shared-memory limit is known to be the largest
     // exact check of a surrogate build: rows recomputed by the path sum
     double sur_tol = 1e-2;                    // rel-L2 above which the model is rebuilt exactly (0: never)
     int sur_check_rows = 512;                 // sampled rows
@@ -239,19 +241,24 @@ void prof_end(lmosem_ctx* c, int cls);
             return ::lmosem::cuda_fail(ctx, e_, "launch at " __FILE__ ":" LMOSEM_STR(__LINE__)); \
     } while (0)
 
-// Lets `kern` be launched with `bytes` of dynamic shared memory.  The limit
+// Lets `kern` be launched with more than 48 KB of dynamic shared memory.  The limit
 // belongs to the function and not to the context, so it is only ever raised, to
 // the most that the function can take: a limit set to each context's own size
-// could be lowered by another host thread between the call and the launch.
+// could be lowered by another host thread between the call and the launch.  (A
+// context asks once per function: 2 us each.)
 template <typename F>
-lmosem_status opt_in_smem(lmosem_ctx* c, F* kern, size_t bytes) {
+lmosem_status opt_in_smem(lmosem_ctx* c, F* kern) {
+    const void* id = reinterpret_cast<const void*>(kern);
+    if (std::find(c->smem_raised.begin(), c->smem_raised.end(), id) != c->smem_raised.end()) return LMOSEM_OK;
     cudaFuncAttributes fa;
     LMOSEM_CK(c, cudaFuncGetAttributes(&fa, kern));
-    if (bytes <= (size_t)fa.maxDynamicSharedSizeBytes) return LMOSEM_OK;
     int dev = 0, most = 0;
     LMOSEM_CK(c, cudaGetDevice(&dev));
     LMOSEM_CK(c, cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    LMOSEM_CK(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes));
+    most -= (int)fa.sharedSizeBytes;
+    if (fa.maxDynamicSharedSizeBytes < most)
+        LMOSEM_CK(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    c->smem_raised.push_back(id);
     return LMOSEM_OK;
 }
 

@@ -1397,8 +1397,8 @@ lmosem_status build_model_rows(lmosem_ctx* c) {
     const size_t smem_w = sizeof(float) * ((size_t)kWOffList + c->n_scat);
     const size_t smem_n = sizeof(float) * ((size_t)kOffList + c->n_scat);
     const size_t smem_t = sizeof(float) * ((size_t)kTOffList + c->n_scat);
-    if ((st = opt_in_smem(c, k_pathsum_tail, smem_t)) || (st = opt_in_smem(c, k_pathsum, smem_w)) ||
-        (st = opt_in_smem(c, k_pathsum_narrow, smem_n)))
+    if ((st = opt_in_smem(c, k_pathsum_tail)) || (st = opt_in_smem(c, k_pathsum)) ||
+        (st = opt_in_smem(c, k_pathsum_narrow)))
         return st;
     // a last column tile with few live columns takes the narrow form
     const int nq_tail = (c->n_sup - (n_ptiles - 1) * kTN + 3) / 4;
@@ -1904,7 +1904,7 @@ lmosem_status build_binned_rows(lmosem_ctx* c, const int32_t* d_rowmap, int n_eb
     B.n_kgroups = (n_ebins + KG - 1) / KG;
     auto kern = KG == 1 ? k_binned<1> : (KG == 2 ? k_binned<2> : k_binned<3>);
     const size_t smem = sizeof(float) * ((size_t)kBOffC + KG * kStage * kTN + kBinWarps + c->n_scat);
-    if ((st = opt_in_smem(c, kern, smem))) return st;
+    if ((st = opt_in_smem(c, kern))) return st;
     // the mass tables of a launch: at most 256 MB
     const int64_t mass_angle = (int64_t)c->n_scat * nb_pad;
     const int msz = (int)std::max<int64_t>(1, std::min<int64_t>(gsz, (int64_t(1) << 26) / std::max<int64_t>(1, mass_angle)));

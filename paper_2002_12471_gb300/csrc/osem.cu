@@ -1166,7 +1166,7 @@ lmosem_status launch_pass_cpa_t(lmosem_ctx* c, PassArgs A, int64_t rows, int nt)
     while (S > 2 && (size_t)S * gbytes > (size_t)smem_max) --S;
     if ((size_t)S * gbytes > (size_t)smem_max) return launch_pass_reg_t<H, VPT, BACK, W>(c, A, rows, nt);
     const size_t smem = (size_t)S * gbytes;
-    if (lmosem_status st = opt_in_smem(c, kern, smem)) return st;
+    if (lmosem_status st = opt_in_smem(c, kern)) return st;
     int per_sm = 0;
     LMOSEM_CK(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem));
     int64_t grid = std::max(1, per_sm) * (int64_t)sms;
@@ -1207,7 +1207,7 @@ lmosem_status launch_pass_t(lmosem_ctx* c, PassArgs A0, int64_t rows, int nt) {
     if ((int64_t)S * G * rb > smem_max)  // two stages of one row do not fit: use the register pass
         return launch_pass_reg_t<H, VPT, BACK, W>(c, A0, rows, nt);
     const size_t smem = (size_t)S * G * rb;
-    if (lmosem_status st = opt_in_smem(c, kern, smem)) return st;
+    if (lmosem_status st = opt_in_smem(c, kern)) return st;
     int per_sm = 0, dev = 0, sms = 0;
     LMOSEM_CK(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem));
     LMOSEM_CK(c, cudaGetDevice(&dev));
@@ -1301,7 +1301,7 @@ lmosem_status launch_coop_t(lmosem_ctx* c, CoopArgs A, int nt) {
     while (S > 2 && (size_t)S * gbytes > (size_t)smem_max) --S;
     if ((size_t)S * gbytes > (size_t)smem_max) return fail(c, LMOSEM_ENOTIMPL, "rows too wide for the ring");
     const size_t smem = (size_t)S * gbytes;
-    if (lmosem_status st = opt_in_smem(c, kern, smem)) return st;
+    if (lmosem_status st = opt_in_smem(c, kern)) return st;
     int per_sm = 0;
     LMOSEM_CK(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem));
     if (per_sm < 1) return fail(c, LMOSEM_ENOTIMPL, "the persistent pass does not fit an SM");
